@@ -91,6 +91,10 @@ struct HessScratch;  // Hessian / Lanczos / MMF scratch (hessian.cu)
 void hess_scratch_destroy(HessScratch *h);
 struct HtstScratch;  // full-spectrum Lanczos scratch (htst.cu)
 void htst_scratch_destroy(HtstScratch *h);
+// Unit eigenvector y of the symmetric tridiagonal matrix (diagonal alpha,
+// couplings beta) for its eigenvalue lam (htst.cu).
+void tri_eigenvector(const std::vector<double> &alpha, const std::vector<double> &beta, double lam,
+                     std::vector<double> &y);
 
 struct sp_ctx {
     int prec = SP_F32;

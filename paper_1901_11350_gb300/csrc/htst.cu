@@ -296,6 +296,8 @@ int tri_eigenvalues(HtstScratch &h, const std::vector<double> &alpha, const std:
     return 0;
 }
 
+}  // namespace
+
 // Eigenvector y (unit) of the tridiagonal for the eigenvalue lam, by inverse
 // iteration with a shift just below lam (tridiagonal LU with partial
 // pivoting).
@@ -355,6 +357,8 @@ void tri_eigenvector(const std::vector<double> &alpha, const std::vector<double>
         for (double &v : y) v /= nr;
     }
 }
+
+namespace {
 
 int setup(sp_ctx *c)
 {
