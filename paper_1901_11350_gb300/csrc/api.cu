@@ -183,11 +183,13 @@ template <typename T> void fill_stencil(const sp_ctx *c, Stencil<T> &S)
                 E.Dz = (T)e.D[2];
                 // i = b + nb (c0 + n0 (c1 + n1 c2)), j the same with jb, c + d
                 E.lin = (e.jb - b) + c->nb * (e.d[0] + c->nc[0] * (e.d[1] + c->nc[1] * e.d[2]));
+                for (int k = 0; k < 3; ++k) E.side |= (e.d[k] < 0 ? 1u : e.d[k] > 0 ? 2u : 0u) << (2 * k);
                 S.r0 = std::max(S.r0, std::abs(e.d[0]));
                 S.r1 = std::max(S.r1, std::abs(e.d[1]));
                 S.r2 = std::max(S.r2, std::abs(e.d[2]));
             }
     }
+    if (S.nb == 1 && (q == 4 || q == 6) && S.r0 <= 1 && S.r1 <= 1 && S.r2 <= 1) S.fixed = q;
 }
 
 // The 27-point fast path applies to a one-atom lattice whose bonds stay in

@@ -63,6 +63,19 @@ template <typename T> __device__ __forceinline__ v3<T> normalised(v3<T> a)
     return r * a;
 }
 
+// Forms whose every rounding is written out: the same bits in whatever kernel
+// they are inlined into (the compiler fuses the plain forms above as it sees
+// fit, which differs between kernels).
+template <typename T> __device__ __forceinline__ T xdot(v3<T> a, v3<T> b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
+template <typename T> __device__ __forceinline__ v3<T> xcross(v3<T> a, v3<T> b)
+{
+    return {fma(a.y, b.z, -(a.z * b.y)), fma(a.z, b.x, -(a.x * b.z)), fma(a.x, b.y, -(a.y * b.x))};
+}
+// v - (v.n) n, and (v.n) n - v
+template <typename T> __device__ __forceinline__ v3<T> tangent(v3<T> v, v3<T> n) { return axpy(-xdot(v, n), n, v); }
+template <typename T> __device__ __forceinline__ v3<T> minus_tangent(v3<T> v, v3<T> n) { return axpy(xdot(v, n), n, -v); }
+template <typename T> __device__ __forceinline__ v3<T> xunit(v3<T> a) { return rnorm(xdot(a, a)) * a; }
+
 __device__ __forceinline__ v3<float> ld(const float4 *p, long i)
 {
     float4 v = __ldg(p + i);
@@ -167,11 +180,14 @@ __device__ __forceinline__ double to_double(f2sum v) { return (double)v.hi + (do
 // ---------------------------------------------------------------- stencil
 // One directed neighbour entry: basis atom jb in cell c + d, exchange J and
 // DMI vector D_ij as seen from the centre atom.
-template <typename T> struct NbrEntry {
-    int jb, d0, d1, d2;
-    int lin;  // j - i for a site whose neighbours need no wrap (see Stencil::r0)
+template <typename T> struct alignas(16) NbrEntry {
     T J, Dx, Dy, Dz;
+    int lin;        // j - i for a site whose neighbours need no wrap (see Stencil::r0)
+    unsigned side;  // bits 0..5: d0 < 0, d0 > 0, d1 < 0, d1 > 0, d2 < 0, d2 > 0
+    int jb, d0, d1, d2;
 };
+// most entries of a stencil whose neighbour loop is unrolled (Stencil::fixed)
+constexpr int kFixedNbr = 6;
 
 // Division of a non-negative int below 2^31 by a fixed positive divisor d
 // as q = (umulhi(n, m) + n) >> s with s = ceil(log2 d) and
@@ -207,6 +223,10 @@ template <typename T> struct alignas(16) Stencil {
     int r0, r1, r2;             // largest |d| of the entries along each direction
     FastDiv fnb, fn0, fn1;      // division by nb, n0, n1
     int off[SP_MAX_BASIS + 1];  // entries of basis b: [off[b], off[b+1])
+    // 4 or 6 entries, one atom per cell, bonds of one cell at most (the square
+    // and the hexagonal plane, the simple cubic lattice): the number of entries,
+    // else 0
+    int fixed;
     T mu[SP_MAX_BASIS];         // mu_b mu_B, meV/T
     T Bz[SP_MAX_BASIS][3];      // Zeeman field mu_b mu_B B, meV
     T K[SP_MAX_BASIS];          // anisotropy K_b, meV
@@ -218,16 +238,21 @@ static_assert(sizeof(Stencil<float>) % 16 == 0 && sizeof(Stencil<double>) % 16 =
 
 // Copy of the part of a stencil in global memory that is in use (header and
 // the entries of every basis atom) into shared memory, by the whole block;
-// the block's later per-neighbour reads then come from shared memory.
+// the block's later per-neighbour reads then come from shared memory.  The
+// header and the first entries are copied before their number is looked at:
+// one trip to memory for the common stencils.
 template <typename T>
 __device__ __forceinline__ void stage_stencil(const Stencil<T> *__restrict__ g, Stencil<T> *s)
 {
-    const int ne = g->off[g->nb];
-    const size_t bytes = offsetof(Stencil<T>, e) + (size_t)ne * sizeof(NbrEntry<T>);
-    const int n16 = (int)((bytes + 15) / 16);
+    constexpr int kFirst = (int)((offsetof(Stencil<T>, e) + kFixedNbr * sizeof(NbrEntry<T>) + 15) / 16);
     const uint4 *src = reinterpret_cast<const uint4 *>(g);
     uint4 *dst = reinterpret_cast<uint4 *>(s);
-    for (int k = threadIdx.x; k < n16; k += blockDim.x) dst[k] = src[k];
+    for (int k = threadIdx.x; k < kFirst; k += blockDim.x) dst[k] = src[k];
+    __syncthreads();
+    const int ne = s->off[s->nb];
+    if (ne <= kFixedNbr) return;
+    const int n16 = (int)((offsetof(Stencil<T>, e) + (size_t)ne * sizeof(NbrEntry<T>) + 15) / 16);
+    for (int k = kFirst + threadIdx.x; k < n16; k += blockDim.x) dst[k] = src[k];
     __syncthreads();
 }
 
@@ -246,12 +271,20 @@ __device__ __forceinline__ int wrap(int x, int n, int per)
 template <typename T>
 __device__ __forceinline__ void decode_site(const Stencil<T> &S, int i, int &b, int &c0, int &c1, int &c2)
 {
-    int r = fdiv(i, S.fnb);
-    b = i - r * S.nb;
+    int r = i;
+    b = 0;
+    if (S.nb > 1) {
+        r = fdiv(i, S.fnb);
+        b = i - r * S.nb;
+    }
     int r1 = fdiv(r, S.fn0);
     c0 = r - r1 * S.n0;
-    c2 = fdiv(r1, S.fn1);
-    c1 = r1 - c2 * S.n1;
+    c2 = 0;
+    c1 = r1;
+    if (S.n2 > 1) {
+        c2 = fdiv(r1, S.fn1);
+        c1 = r1 - c2 * S.n1;
+    }
 }
 
 // Local part of B_eff = -dH/dn at spin i (Eq. 1 without the dipole term):
@@ -282,23 +315,131 @@ __device__ __forceinline__ int nbr_index(const Stencil<T> &S, const NbrEntry<T> 
     return E.jb + S.nb * (x0 + S.n0 * (x1 + S.n1 * x2));
 }
 
+// The stencil entries of basis atom b at site i = (b, c0, c1, c2), in order:
+// use(E, v) with v = load(j) for every entry whose neighbour j exists.
+//
+// What bounds the per-spin passes is the number of instructions they issue
+// (ncu, 1024 x 1024 hexagonal plane: 622 a spin in the Depondt predictor, 80%
+// of the issue slots, with a loop over the entries; 470 with this one and the
+// rotation without square root and division, 784 -> 589 us for 20 steps).  So the stencils that are used most, NE entries of one
+// atom per cell, have a loop without indices: the couplings are operands from
+// the constant bank (or from shared memory at fixed addresses) and the loads
+// are in flight together.  At an edge the wrap is one correction of i + lin
+// per side, computed once per site, and nothing is fetched across an open
+// side.
+template <int NE, typename T, typename Load, typename Use>
+__device__ __forceinline__ void fixed_neighbours(const Stencil<T> &S, int i, int c0, int c1, int c2, Load load, Use use)
+{
+    v3<T> v[NE];
+    if (interior_site(S, c0, c1, c2)) {
+#pragma unroll
+        for (int k = 0; k < NE; ++k) v[k] = load(i + S.e[k].lin);
+#pragma unroll
+        for (int k = 0; k < NE; ++k) use(S.e[k], v[k]);
+    } else {
+        const int s1 = S.n0 * S.n1;
+        const bool lo0 = c0 == 0, hi0 = c0 == S.n0 - 1, lo1 = c1 == 0, hi1 = c1 == S.n1 - 1, lo2 = c2 == 0,
+                   hi2 = c2 == S.n2 - 1;
+        const unsigned w[6] = {lo0 ? (unsigned)S.n0 : 0u,  hi0 ? 0u - (unsigned)S.n0 : 0u,
+                               lo1 ? (unsigned)s1 : 0u,    hi1 ? 0u - (unsigned)s1 : 0u,
+                               lo2 ? (unsigned)S.N : 0u,   hi2 ? 0u - (unsigned)S.N : 0u};
+        const unsigned open = (S.per0 ? 0u : (lo0 ? 1u : 0u) | (hi0 ? 2u : 0u)) |
+                              (S.per1 ? 0u : (lo1 ? 4u : 0u) | (hi1 ? 8u : 0u)) |
+                              (S.per2 ? 0u : (lo2 ? 16u : 0u) | (hi2 ? 32u : 0u));
+#pragma unroll
+        for (int k = 0; k < NE; ++k) {
+            unsigned j = (unsigned)(i + S.e[k].lin);
+            const unsigned side = S.e[k].side;
+#pragma unroll
+            for (int d = 0; d < 6; ++d)
+                if (side & (1u << d)) j += w[d];
+            if (!(side & open)) v[k] = load((int)j);
+        }
+#pragma unroll
+        for (int k = 0; k < NE; ++k)
+            if (!(S.e[k].side & open)) use(S.e[k], v[k]);
+    }
+}
+
+template <typename T, typename Load, typename Use>
+__device__ __forceinline__ void for_neighbours(const Stencil<T> &S, int i, int b, int c0, int c1, int c2, Load load,
+                                               Use use)
+{
+    if (S.fixed == 6) {
+        fixed_neighbours<6>(S, i, c0, c1, c2, load, use);
+    } else if (S.fixed == 4) {
+        fixed_neighbours<4>(S, i, c0, c1, c2, load, use);
+    } else {
+        const bool inner = interior_site(S, c0, c1, c2);
+        for (int q = S.off[b]; q < S.off[b + 1]; ++q) {
+            const int j = nbr_index(S, S.e[q], i, inner, c0, c1, c2);
+            if (j >= 0) use(S.e[q], load(j));
+        }
+    }
+}
+
+// B + J v + v x D.  FP32: the cross product first, one rounding of it and one
+// of the product with J at the magnitude of the field.
+__device__ __forceinline__ v3<float> add_bond(const NbrEntry<float> &E, v3<float> v, v3<float> B)
+{
+    return {fmaf(E.J, v.x, __fadd_rn(B.x, fmaf(v.y, E.Dz, -__fmul_rn(v.z, E.Dy)))),
+            fmaf(E.J, v.y, __fadd_rn(B.y, fmaf(v.z, E.Dx, -__fmul_rn(v.x, E.Dz)))),
+            fmaf(E.J, v.z, __fadd_rn(B.z, fmaf(v.x, E.Dy, -__fmul_rn(v.y, E.Dx))))};
+}
+__device__ __forceinline__ v3<double> add_bond(const NbrEntry<double> &E, v3<double> v, v3<double> B)
+{
+    return {fma(-v.z, E.Dy, fma(v.y, E.Dz, fma(E.J, v.x, B.x))),
+            fma(-v.x, E.Dz, fma(v.z, E.Dx, fma(E.J, v.y, B.y))),
+            fma(-v.y, E.Dx, fma(v.x, E.Dy, fma(E.J, v.z, B.z)))};
+}
+
+// The on-site field mu_i B + 2 K (Khat.n_i) Khat of basis atom b.
+template <typename T> __device__ __forceinline__ v3<T> onsite_field(const Stencil<T> &S, int b, v3<T> ni)
+{
+    auto at = [&](int a) {
+        T kn = xdot(mk(S.Kh[a][0], S.Kh[a][1], S.Kh[a][2]), ni);
+        T k2 = T(2) * S.K[a] * kn;
+        return mk(fma(k2, S.Kh[a][0], S.Bz[a][0]), fma(k2, S.Kh[a][1], S.Bz[a][1]), fma(k2, S.Kh[a][2], S.Bz[a][2]));
+    };
+    return S.nb == 1 ? at(0) : at(b);  // one atom: operands at fixed addresses
+}
+
 template <typename T, typename R>
 __device__ __forceinline__ v3<T> local_field(const Stencil<T> &S, const R *n, int i, v3<T> ni, int &b)
 {
     int c0, c1, c2;
     decode_site(S, i, b, c0, c1, c2);
-    T kn = dot(mk(S.Kh[b][0], S.Kh[b][1], S.Kh[b][2]), ni);
-    T k2 = T(2) * S.K[b] * kn;
-    v3<T> B = mk(fma(k2, S.Kh[b][0], S.Bz[b][0]), fma(k2, S.Kh[b][1], S.Bz[b][1]), fma(k2, S.Kh[b][2], S.Bz[b][2]));
-    const bool inner = interior_site(S, c0, c1, c2);
-    for (int q = S.off[b]; q < S.off[b + 1]; ++q) {
-        const NbrEntry<T> &E = S.e[q];
-        int j = nbr_index(S, E, i, inner, c0, c1, c2);
-        if (j < 0) continue;
-        v3<T> nj = ld(n, j);
-        v3<T> c = cross(nj, mk(E.Dx, E.Dy, E.Dz));
-        B = axpy(E.J, nj, B + c);
-    }
+    v3<T> B = onsite_field(S, b, ni);
+    for_neighbours(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
+                   [&](const NbrEntry<T> &E, v3<T> v) { B = add_bond(E, v, B); });
+    return B;
+}
+
+// The same with the sum over the bonds compensated (two_sum): the field as
+// hi + lo, in FP32 to the rounding of the bonds' own terms.  In a region where
+// all spins are alike every one of them makes the same rounding error, and the
+// errors of an image's energy do not average out; the energy differences of
+// neighbouring images, which weigh the tangents, are small against it.
+__device__ __forceinline__ void compensate(float t, float &hi, float &lo)
+{
+    const f2sum s = two_sum(hi, t);
+    hi = s.hi;
+    lo += s.lo;
+}
+template <typename R>
+__device__ __forceinline__ v3<float> local_field_comp(const Stencil<float> &S, const R *n, int i, v3<float> ni, int &b,
+                                                      v3<float> &lo)
+{
+    int c0, c1, c2;
+    decode_site(S, i, b, c0, c1, c2);
+    v3<float> B = onsite_field(S, b, ni), l = mk(0.f, 0.f, 0.f);
+    for_neighbours(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
+                   [&](const NbrEntry<float> &E, v3<float> v) {
+                       compensate(fmaf(E.J, v.x, fmaf(v.y, E.Dz, -__fmul_rn(v.z, E.Dy))), B.x, l.x);
+                       compensate(fmaf(E.J, v.y, fmaf(v.z, E.Dx, -__fmul_rn(v.x, E.Dz))), B.y, l.y);
+                       compensate(fmaf(E.J, v.z, fmaf(v.x, E.Dy, -__fmul_rn(v.y, E.Dx))), B.z, l.z);
+                   });
+    lo = l;
     return B;
 }
 
@@ -407,24 +548,55 @@ template <typename T> __device__ __forceinline__ v3<T> llg_A(T c, T alpha, v3<T>
     return c * axpy(alpha, cross(n, B), B);
 }
 
-// Depondt step: rotate n about -Ahat by |A| dt (Rodrigues' formula).
+// Depondt step: rotate n about -Ahat by th = |A| dt (Rodrigues' formula),
+//   n cos th - (A x n) dt sin(th)/th + A (A.n) dt^2 (1 - cos th)/th^2.
+// Both quotients are even in th: for th^2 <= 1/4 (a step turns a spin by
+// hundredths of a radian) they are summed as Taylor series in th^2, to below
+// half a unit in the last place, and neither |A| nor a division is needed.
 __device__ __forceinline__ void sincos_(float x, float *s, float *c) { sincosf(x, s, c); }
 __device__ __forceinline__ void sincos_(double x, double *s, double *c) { sincos(x, s, c); }
+// sin(th)/th and (1 - cos th)/th^2 for t = th^2 <= 1/4
+__device__ __forceinline__ void rotation_series(float t, float *s, float *c)
+{
+    *s = fmaf(t, fmaf(t, fmaf(t, -1.f / 5040.f, 1.f / 120.f), -1.f / 6.f), 1.f);
+    *c = fmaf(t, fmaf(t, fmaf(t, -1.f / 40320.f, 1.f / 720.f), -1.f / 24.f), 0.5f);
+}
+__device__ __forceinline__ void rotation_series(double t, double *s, double *c)
+{
+    double a = -1.0 / 1307674368000.0, b = 1.0 / 20922789888000.0 * -1.0;
+    a = fma(t, a, 1.0 / 6227020800.0);
+    b = fma(t, b, 1.0 / 87178291200.0);
+    a = fma(t, a, -1.0 / 39916800.0);
+    b = fma(t, b, -1.0 / 479001600.0);
+    a = fma(t, a, 1.0 / 362880.0);
+    b = fma(t, b, 1.0 / 3628800.0);
+    a = fma(t, a, -1.0 / 5040.0);
+    b = fma(t, b, -1.0 / 40320.0);
+    a = fma(t, a, 1.0 / 120.0);
+    b = fma(t, b, 1.0 / 720.0);
+    a = fma(t, a, -1.0 / 6.0);
+    b = fma(t, b, -1.0 / 24.0);
+    *s = fma(t, a, 1.0);
+    *c = fma(t, b, 0.5);
+}
 template <typename T> __device__ __forceinline__ v3<T> rotate(v3<T> n, v3<T> A, T dt)
 {
-    T w2 = dot(A, A);
+    const T w2 = xdot(A, A), t = w2 * (dt * dt);
     if (w2 == T(0)) return n;
-    T iw = rnorm(w2);
-    T th = w2 * iw * dt;
-    v3<T> ax = (-iw) * A;
-    T s, c;
-    sincos_(th, &s, &c);
-    v3<T> axn = cross(ax, n);
-    T an = dot(ax, n);
-    // 1 - cos without cancellation for small angles: sin^2 / (1 + cos)
-    T omc = c > T(0) ? s * s / (T(1) + c) : T(1) - c;
-    // n cos + (ax x n) sin + ax (ax.n)(1 - cos)
-    return axpy(an * omc, ax, axpy(s, axn, c * n));
+    T s, c, cs;
+    if (t <= T(0.25)) {
+        rotation_series(t, &s, &c);
+        cs = fma(-t, c, T(1));  // cos th
+        s *= dt;
+        c *= dt * dt;
+    } else {
+        const T iw = rnorm(w2), th = w2 * iw * dt;
+        sincos_(th, &s, &cs);
+        // 1 - cos without cancellation for small angles: sin^2 / (1 + cos)
+        c = (cs > T(0) ? s * s / (T(1) + cs) : T(1) - cs) * iw * iw;
+        s *= iw;
+    }
+    return axpy(c * xdot(A, n), A, axpy(-s, xcross(A, n), cs * n));
 }
 
 // SIB step (Appendix C): the solution of M x = M^T n with M = I + skew(a),

@@ -23,6 +23,13 @@
 #define SPGB_LLG_PDL 1
 #endif
 
+// blocks of 256 per SM the FP32 passes' register allocation is held to (512 x
+// 512 hexagonal plane with the dipole field, 20 steps: 6: 1290 us, 5: 1322, 4:
+// 1340; 1024 x 1024 without: 589, 588, 621)
+#ifndef SPGB_LLG_MINB
+#define SPGB_LLG_MINB 6
+#endif
+
 namespace spgb {
 
 // ---------------------------------------------------------------- field
@@ -103,7 +110,7 @@ __device__ __forceinline__ void corr_spin(const Stencil<T> &S, R *n, const R *np
 }
 
 template <typename T, int SOLVER>
-__global__ void __launch_bounds__(kBlock) k_llg_pred(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ n,
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_llg_pred(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ n,
                                                      const rec_t<T> *__restrict__ Bdd, rec_t<T> *__restrict__ np,
                                                      rec_t<T> *__restrict__ q, const LlgConst<T> c)
 {
@@ -117,7 +124,7 @@ __global__ void __launch_bounds__(kBlock) k_llg_pred(const __grid_constant__ Ste
 }
 
 template <typename T, int SOLVER>
-__global__ void __launch_bounds__(kBlock) k_llg_corr(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n,
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_llg_corr(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n,
                                                      const rec_t<T> *__restrict__ np, const rec_t<T> *__restrict__ q,
                                                      const rec_t<T> *__restrict__ Bdd, const LlgConst<T> c)
 {

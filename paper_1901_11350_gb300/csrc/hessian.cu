@@ -294,18 +294,14 @@ __device__ __forceinline__ v3<T> lz_product(const Stencil<T> &S, const rec_t<T> 
 {
     int bs, c0, c1, c2;
     decode_site(S, i, bs, c0, c1, c2);
-    const bool inner = interior_site(S, c0, c1, c2);
     const v3<T> kh = mk(S.Kh[bs][0], S.Kh[bs][1], S.Kh[bs][2]);
     v3<T> L = (T(2) * S.K[bs] * dot(kh, u)) * kh;
-    for (int e = S.off[bs]; e < S.off[bs + 1]; ++e) {
-        const NbrEntry<T> &E = S.e[e];
-        const int j = nbr_index(S, E, i, inner, c0, c1, c2);
-        if (j < 0) continue;
-        const v3<T> v = ldg2(w, j);  // tangent already: no projection here
-        L.x = fma(-v.z, E.Dy, fma(v.y, E.Dz, fma(E.J, v.x, L.x)));
-        L.y = fma(-v.x, E.Dz, fma(v.z, E.Dx, fma(E.J, v.y, L.y)));
-        L.z = fma(-v.y, E.Dx, fma(v.x, E.Dy, fma(E.J, v.z, L.z)));
-    }
+    for_neighbours(S, i, bs, c0, c1, c2, [&](int j) { return ldg2(w, j); },  // tangent already: no projection here
+                   [&](const NbrEntry<T> &E, v3<T> v) {
+                       L.x = fma(-v.z, E.Dy, fma(v.y, E.Dz, fma(E.J, v.x, L.x)));
+                       L.y = fma(-v.x, E.Dz, fma(v.z, E.Dx, fma(E.J, v.y, L.y)));
+                       L.z = fma(-v.y, E.Dx, fma(v.x, E.Dy, fma(E.J, v.z, L.z)));
+                   });
     return axpy(nB, u, axpy(dot(L, ni), ni, -L));
 }
 

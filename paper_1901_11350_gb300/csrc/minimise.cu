@@ -7,12 +7,21 @@
 // reduced deterministically: every block writes its partial, and the last
 // block of the image to finish (atomic ticket) sums the image's partials in
 // a fixed order and re-arms the ticket.  Kernels of one iteration:
-//   move    v <- projection of v on F (from the previous force pass),
+//   move    v = c F, c = v.F / F.F or 0 from the previous force pass,
 //           x <- normalise(x + dt v + dt^2/(2m) F)          (interior images)
-//   field   B(x), E_v, Pg = -(B - (B.x)x), theta^2 to image v+1
-//   tangent improved tangent, per-spin projection, |tau|^2, Pg.tau
-//   force   F' (spring / climbing image), v <- v + dt/(2m)(F + F'),
-//           v.F', F'.F', max |F'|
+//   field   B(x), E_v, Pg = -(B - (B.x)x), theta^2 to image v+1, and the
+//           products of the differences d+ and d- to the neighbouring images
+//           with each other and with Pg
+//   coefs   per chain, from its images' sums: tangent weights, |tau|^2,
+//           Pg.tau, the climbing image, force coefficients a
+//   force   tau = P(w+ d+ + w- d-), F' = -Pg + a tau, v.F', F'.F', max |F'| with v = c F + dt/(2m)(F + F')
+// What bounds them: memory.  The projected velocity is a multiple of F, so no
+// pass stores it (the call's last one does), and tau is formed again in the
+// force pass rather than stored: 144 B per spin and iteration.  |tau|^2 and
+// Pg.tau follow from the field pass's products (tau is linear in the weights).
+// 3.6 M spins in 12 chains: 335 -> 240 us an iteration (with tau and v stored,
+// 288 B, and a neighbour loop with indices).  The field pass is 55% of it and
+// bound by the instructions it issues (830 a spin, 61% of the issue slots).
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
@@ -29,17 +38,20 @@ struct ImgInfo {
     long long spin0;  // record offset of image 0 of the chain
     int N, chain, nu, M, g0, blk0, bpi;
     int kind;  // SP_IMAGE_* or -1: climbing decided by the climbing flag
+    int spt;   // spins per thread (GNEB passes; 1 elsewhere)
 };
-struct BlkInfo {
-    int g, t;
+struct alignas(16) BlkInfo {
+    int g, t, chain;  // image, block of the image, the image's chain
 };
 
 // per-image scalar slots (kS doubles per image): energy, squared geodesic
-// distance to the next image, |tau|^2, Pg.tau, v.F, F.F, max_i |F_i|^2,
-// energy-weighted segment length, tangent weights of the forward and
-// backward differences, force coefficient a (F = -Pg + a tau), velocity
-// projection coefficient v.F / F.F
-enum { kE = 0, kL2, kTT, kGT, kVF, kFF, kFMAX, kLW, kWP, kWM, kA, kC, kS = 16 };
+// distance to the next image, products d+.d+, d+.d-, d-.d-, Pg.d+, Pg.d- of
+// the projected differences to the next and the previous image, v.F, F.F,
+// max_i |F_i|^2, energy-weighted segment length, tangent weights of the
+// forward and backward differences, |tau|^2, Pg.tau, force coefficient a
+// (F = -Pg + a tau), velocity projection coefficient v.F / F.F, max |F|
+// (minimiser)
+enum { kE = 0, kL2, kPP, kPM, kMM, kGP, kGM, kVF, kFF, kFMAX, kLW, kWP, kWM, kTT, kGT, kA, kC, kFN, kS = 18 };
 
 struct Buf {
     void *p = nullptr;
@@ -60,7 +72,7 @@ int grow(Buf &b, size_t bytes)
 }  // namespace
 
 struct MinScratch {
-    Buf F, G, Tau, scal, part, cnt, blk, img, sten, state, aux, sync;
+    Buf F, G, scal, part, cnt, blk, img, sten, state, aux, sync;
     int *host_state = nullptr;  // pinned: iters, active
     double *host_fmax = nullptr;
     // batch layout last uploaded (block/image tables and stencils)
@@ -74,11 +86,20 @@ struct MinScratch {
 };
 
 constexpr int kGraphIters = 8;
+constexpr int kPartRow = 8;  // doubles of a block's partials, at most
+// blocks per SM the register allocation is held to (FP32): GNEB field pass 4
+// (240 us an iteration; 3: 246, 2: 274)
+#ifndef SPGB_VP_MINB
+#define SPGB_VP_MINB 6
+#endif
+#ifndef SPGB_GF_MINB
+#define SPGB_GF_MINB 4
+#endif
 
 void min_scratch_destroy(MinScratch *s)
 {
     if (!s) return;
-    Buf *bufs[] = {&s->F, &s->G, &s->Tau, &s->scal, &s->part, &s->cnt, &s->blk, &s->img, &s->sten, &s->state, &s->aux,
+    Buf *bufs[] = {&s->F, &s->G, &s->scal, &s->part, &s->cnt, &s->blk, &s->img, &s->sten, &s->state, &s->aux,
                    &s->sync};
     for (Buf *b : bufs)
         if (b->p) cudaFree(b->p);
@@ -121,117 +142,211 @@ template <typename T> struct Acc {
 template <> struct Acc<float> {
     using type = f2sum;
 };
-__device__ __forceinline__ f2sum acc_dot(v3<float> a, v3<float> b) { return exact_dot(a, b); }
-__device__ __forceinline__ double acc_dot(v3<double> a, v3<double> b) { return dot(a, b); }
-
-template <int NV, typename V>
-__device__ __forceinline__ V combine(int k, unsigned maxmask, V a, V b)
+// exact_dot and exact_square with products that no addition is fused with
+__device__ __forceinline__ f2sum acc_prod(float a, float b)
 {
-    return ((maxmask >> k) & 1u) ? nan_max(a, b) : a + b;
+    const float p = __fmul_rn(a, b);
+    return {p, fmaf(a, b, -p)};
+}
+__device__ __forceinline__ f2sum acc_dot(v3<float> a, v3<float> b)
+{
+    return acc_prod(a.x, b.x) + acc_prod(a.y, b.y) + acc_prod(a.z, b.z);
+}
+__device__ __forceinline__ double acc_prod(double a, double b) { return __dmul_rn(a, b); }
+// r += a.b for a sum of a few spins: the products and the errors of the
+// additions to r.hi go to r.lo one after another
+__device__ __forceinline__ void acc_add(f2sum &r, float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    const f2sum s = two_sum(r.hi, p);
+    r.hi = s.hi;
+    r.lo += s.lo + fmaf(a, b, -p);
+}
+__device__ __forceinline__ void acc_add(f2sum &r, v3<float> a, v3<float> b)
+{
+    acc_add(r, a.x, b.x);
+    acc_add(r, a.y, b.y);
+    acc_add(r, a.z, b.z);
+}
+__device__ __forceinline__ void acc_add(double &r, double a, double b) { r = fma(a, b, r); }
+__device__ __forceinline__ double acc_dot(v3<double> a, v3<double> b) { return xdot(a, b); }
+__device__ __forceinline__ void acc_add(double &r, v3<double> a, v3<double> b) { r += xdot(a, b); }
+
+__device__ __forceinline__ float xor_of(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double xor_of(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ f2sum xor_of(f2sum v, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
 }
 
-struct NoPost {
-    __device__ void operator()(double *) const {}
-};
-
-// Deterministic per-image reduction of NV values (bit k of maxmask: max
-// instead of sum; maxima are of non-negative values, 0 is their identity).
-// Every thread of every block of the image must call it.  The warp-level
-// step runs in the values' own type V (float, double or f2sum); from the warp
-// results on everything is FP64.  After one barrier warps 1.. leave; warp 0
-// combines the warp results by a fixed shuffle tree into the block's partial
-// and takes a ticket; warp 0 of the image's last block sums the partials
-// (lane l takes partials l, l + 32, ..., then a shuffle tree), writes the
-// totals to out[] and calls post(out).
-template <int NV, typename V, typename Post = NoPost>
-__device__ void image_reduce(V (&v)[NV], unsigned maxmask, double *__restrict__ part, int blk, int blk0, int bpi,
-                             unsigned *counter, double *out, Post post = Post())
+// Sums over a warp of NS values per lane (a power of two); the 32 / NS lanes
+// l with l NS / 32 = k receive the sum of value k.  Each step halves the
+// values a lane carries: NS - 1 additions and one more per step that is left,
+// not five per value.
+template <int NS, typename V> __device__ __forceinline__ V warp_sums(V (&v)[NS])
 {
-    constexpr int NW = kBlock / 32;
-    static_assert(NW <= 32, "one warp combines the warp results");
-    __shared__ double sh[NW][NV];
+    const int l = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] = combine<NV>(k, maxmask, v[k], shfl_down(v[k], o));
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0)
-        for (int k = 0; k < NV; ++k) sh[w][k] = to_double(v[k]);
+    for (int n = NS / 2; n > 0; n >>= 1, o >>= 1) {
+        const bool up = (l & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const V send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + xor_of(send, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) v[0] = v[0] + xor_of(v[0], o);
+    return v[0];
+}
+
+// The type a block's sums are combined in: float-float for float.
+template <typename V> struct Wide {
+    using type = V;
+};
+template <> struct Wide<float> {
+    using type = f2sum;
+};
+__device__ __forceinline__ f2sum widen(float v) { return {v, 0.f}; }
+__device__ __forceinline__ f2sum widen(f2sum v) { return v; }
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// Deterministic per-image reduction of NS sums (2 or 8) and, with MAX, one
+// maximum (of non-negative values).  Every thread of every block of the image
+// must call it.  The block's sums run in the values' own type V (float, double
+// or f2sum), the image's in FP64.  After one
+// barrier warps 1.. leave; warp 0 combines the warp results by a fixed shuffle
+// tree into the block's partials and takes a ticket; warp 0 of the image's
+// last block sums the partials in a fixed order, writes the totals to
+// out[0..NS) (and out[NS]) and calls post(lane).
+template <int NS, bool MAX, typename V, typename Post>
+__device__ __forceinline__ void image_sums(V (&v)[NS], V m, double *__restrict__ part, int blk, int blk0, int bpi,
+                                           unsigned *counter, double *out, Post post)
+{
+    constexpr int NW = kBlock / 32, LPV = 32 / NS, ROW = MAX ? 4 : 8, NV = NS + (MAX ? 1 : 0);
+    static_assert(NV <= ROW && ROW <= kPartRow, "a row holds the values");
+    // (the block's own sums in V, float-float for float: a conversion to FP64 per
+    // warp and value was a fifth of the time of a minimiser's force pass)
+    using W = typename Wide<V>::type;
+    __shared__ V sh[NW][NV];
+    const V s = warp_sums(v);
+    if (MAX)
+        for (int o = 16; o > 0; o >>= 1) m = nan_max(m, shfl_down(m, o));
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (l % LPV == 0) sh[w][l / LPV] = s;
+    if (MAX && l == 0) sh[w][NS] = m;
     __syncthreads();
     if (w != 0) return;
-    double a[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        a[k] = l < NW ? sh[l][k] : 0.0;
-        for (int o = NW / 2; o > 0; o >>= 1) a[k] = combine<NV, double>(k, maxmask, a[k], shfl_down(a[k], o));
+    W t{};
+    for (int k = l % LPV; k < NW; k += LPV) t = t + widen(sh[k][l / LPV]);
+    for (int o = LPV / 2; o > 0; o >>= 1) t = t + xor_of(t, o);
+    const double a = to_double(t);
+    double mx = 0.0;
+    if (MAX) {
+        V mv = l < NW ? sh[l][NS] : V{};
+        for (int o = NW / 2; o > 0; o >>= 1) mv = nan_max(mv, shfl_down(mv, o));
+        mx = to_double(mv);
     }
+    if (l % LPV == 0) part[(size_t)blk * ROW + l / LPV] = a;
+    if (MAX && l == 0) part[(size_t)blk * ROW + NS] = mx;
+    __threadfence();
+    __syncwarp();
     int last = 0;
-    if (l == 0) {
-        for (int k = 0; k < NV; ++k) part[(size_t)blk * NV + k] = a[k];
-        __threadfence();
-        unsigned ticket = atomicAdd(counter, 1u);
-        last = ticket == (unsigned)(bpi - 1);
-    }
+    if (l == 0) last = atomicAdd(counter, 1u) == (unsigned)(bpi - 1);
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
-    double acc[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-    for (int p = l; p < bpi; p += 32)
-        for (int k = 0; k < NV; ++k)
-            acc[k] = combine<NV, double>(k, maxmask, acc[k], __ldcg(&part[(size_t)(blk0 + p) * NV + k]));
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
-        for (int o = 16; o > 0; o >>= 1) acc[k] = combine<NV, double>(k, maxmask, acc[k], shfl_down(acc[k], o));
-    if (l == 0) {
-        for (int k = 0; k < NV; ++k) out[k] = acc[k];
-        post(out);
-        atomicExch(counter, 0u);
+    const int k = l % ROW;
+    const bool is_max = MAX && k == NS;
+    double acc = 0.0;
+    if (k < NV)
+        for (int p = l / ROW; p < bpi; p += 32 / ROW) {
+            const double x = __ldcg(&part[(size_t)(blk0 + p) * ROW + k]);
+            acc = is_max ? nan_max(acc, x) : acc + x;
+        }
+    for (int o = 16; o >= ROW; o >>= 1) {
+        const double x = xor_of(acc, o);
+        acc = is_max ? nan_max(acc, x) : acc + x;
     }
+    if (l < NV) out[l] = acc;
+    __threadfence();
+    __syncwarp();
+    if (l == 0) atomicExch(counter, 0u);
+    post(l);
 }
 
 // After a force pass (out = scal + kS g + kVF): the projection coefficient
-// v.F / F.F (0 unless both are positive) of the next move.
-struct ProjectionPost {
-    __device__ void operator()(double *out) const
+// v.F / F.F (0 unless both are positive) of the next move, and max |F|.
+struct ForcePost {
+    double *out;
+    __device__ void operator()(int l) const
     {
-        double vf = out[kVF - kVF], ff = out[kFF - kVF];
+        if (l != 0) return;
+        const double vf = out[0], ff = out[kFF - kVF];
         out[kC - kVF] = (vf > 0 && ff > 0) ? vf / ff : 0.0;
+        out[kFN - kVF] = sqrt(out[kFMAX - kVF]);
     }
 };
 
 // ============================================================ VP minimiser
 // state (ints): [0] iterations performed, [1] active flag
-// scal (doubles): v.F, F.F, max|F|^2, projection-valid flag
+// scal (doubles): the image slots kVF.. and, at kVP, whether the last force
+// pass had a velocity.
 // (max |F|^2 rather than max |F|: one square root per image instead of one
 // per spin; sqrt is monotonic and correctly rounded, so sqrt(max |F|^2) is
 // exactly max |F| in FP64)
+// Between two force passes the velocity is a multiple c F of the force, so
+// neither pass stores it; the last move of a call does.
+constexpr int kVP = 0;  // slot kE, which the minimiser does not use
+
+// Force pass of spin p = i of a system; mode 0: F only; 1: v from memory (the
+// call's first iteration); 2: v = c F, c the projection coefficient of the
+// previous force pass (read before this block's ticket, so before the
+// system's last block replaces it).
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_vp_force(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ x,
-                                                     rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
+__device__ __forceinline__ void vp_force(const Stencil<T> &S, const rec_t<T> *x, const rec_t<T> *v, rec_t<T> *F, int i,
+                                         T dth_m, int mode, T c, T (&r)[2], T &mx)
+{
+    int b;
+    const v3<T> ni = ld(x, i);
+    const v3<T> B = local_field(S, x, i, ni, b);
+    const v3<T> Fn = tangent(B, ni);
+    if (mode) {
+        const v3<T> Fo = ldc((const rec_t<T> *)F, i);
+        const v3<T> vi = axpy(dth_m, Fo + Fn, mode == 1 ? ldc(v, i) : c * Fo);
+        r[0] = xdot(vi, Fn);
+    }
+    st(F, i, Fn);
+    r[1] = xdot(Fn, Fn);
+    mx = r[1];
+}
+
+// Move of spin i (done: none); last: the projected velocity is stored.
+template <typename T>
+__device__ __forceinline__ void vp_move(rec_t<T> *x, rec_t<T> *v, const rec_t<T> *F, int i, T dt, T dt2_2m, bool proj,
+                                        T c, bool done, bool last)
+{
+    if (done && !last) return;
+    const v3<T> Fi = ldc(F, i), vi = proj ? c * Fi : ldc((const rec_t<T> *)v, i);
+    if (last && proj) st(v, i, vi);
+    if (!done) st(x, i, xunit(axpy(dt2_2m, Fi, axpy(dt, vi, ldc((const rec_t<T> *)x, i)))));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_vp_force(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ x,
+                                                     const rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
                                                      int mode, double *part, unsigned *cnt, double *scal,
                                                      const int *state)
 {
     allow_dependents();
     wait_prerequisite();  // state, scalars and records come from the kernels before
-    if (mode == 1 && state[1] == 0) return;
-    int i = blockIdx.x * kBlock + threadIdx.x;
-    T r[3] = {0, 0, 0};
-    if (i < S.N) {
-        int b;
-        v3<T> ni = ld(x, i);
-        v3<T> B = local_field(S, x, i, ni, b);
-        v3<T> Fn = B - dot(B, ni) * ni;
-        if (mode == 1) {
-            v3<T> vi = axpy(dth_m, ldc(F, i) + Fn, ldc(v, i));
-            st(v, i, vi);
-            r[0] = dot(vi, Fn);
-        }
-        st(F, i, Fn);
-        r[1] = dot(Fn, Fn);
-        r[2] = r[1];
-    }
-    image_reduce<3>(r, 4u, part, blockIdx.x, 0, gridDim.x, cnt, scal);
-    if (blockIdx.x == 0 && threadIdx.x == 0) scal[3] = mode;
+    if (mode && state[1] == 0) return;
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    const T c = mode == 2 ? (T)scal[kC] : T(0);
+    T r[2] = {0, 0}, mx = 0;
+    if (i < S.N) vp_force(S, x, v, F, i, dth_m, mode, c, r, mx);
+    image_sums<2, true>(r, mx, part, blockIdx.x, 0, gridDim.x, cnt, scal + kVF, ForcePost{scal + kVF});
+    if (blockIdx.x == 0 && threadIdx.x == 0) scal[kVP] = mode;
 }
 
 template <typename T>
@@ -241,28 +356,9 @@ __global__ void __launch_bounds__(kBlock) k_vp_move(int N, rec_t<T> *__restrict_
 {
     allow_dependents();
     wait_prerequisite();  // state, scalars and records come from the kernels before
-    __shared__ T s_c;
-    __shared__ int s_done;
-    if (threadIdx.x == 0) {
-        double vf = scal[0], ff = scal[1];
-        s_c = (vf > 0 && ff > 0) ? (T)(vf / ff) : T(0);
-        s_done = (sqrt(scal[2]) < tol) || (k >= max_iter);
-    }
-    __syncthreads();
-    bool done = s_done;
-    bool proj = scal[3] != 0.0;
-    int i = blockIdx.x * kBlock + threadIdx.x;
-    if (i < N) {
-        v3<T> vi;
-        if (proj) {
-            T c = s_c;
-            vi = c * ldc(F, i);
-            st(v, i, vi);
-        } else {
-            vi = ldc(v, i);
-        }
-        if (!done) st(x, i, normalised(axpy(dt2_2m, ldc(F, i), axpy(dt, vi, ldc(x, i)))));
-    }
+    const bool done = scal[kFN] < tol || k >= max_iter;
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    if (i < N) vp_move(x, v, F, i, dt, dt2_2m, scal[kVP] != 0.0, (T)scal[kC], done, k >= max_iter);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         state[1] = done ? 0 : 1;
         if (!done) state[0] = k + 1;
@@ -277,62 +373,28 @@ __global__ void __launch_bounds__(kBlock) k_vp_move(int N, rec_t<T> *__restrict_
 // per-pass kernels: spins by the read-only path) or the plain-load record
 // type of ShRec<T> (the persistent kernel, which reads what other blocks
 // wrote earlier in the same launch).
-template <typename T, typename R>
-__device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                             const Stencil<T> *__restrict__ S, const R *x, R *G, double *part,
-                                             unsigned *cnt, double *scal)
+
+// Spins per thread of a chain's passes: the reductions at the end of a block
+// cost as much as two spins, so long chains share them among four; a chain
+// with fewer blocks than two per SM of 256 spins each is spread out instead.
+// It depends on the chain alone: a chain gets the same sums in any batch.
+inline int gneb_spt(long long spins)
 {
-    BlkInfo bi = blk[vb];
-    ImgInfo im = img[bi.g];
-    // the chain's stencil, staged in shared memory for the neighbour loop
-    __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
-    Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
-    stage_stencil(S + im.chain, &St);
-    int i = bi.t * kBlock + threadIdx.x;
-    const R *xb = x + im.spin0 + (long long)im.nu * im.N;
-    // energy and squared angle sums: FP64, or float-float for FP32 (the
-    // same sums of the same products to ~1e-14, off the FP64 pipe)
-    using A = typename Acc<T>::type;
-    A r[2] = {A{}, A{}};
-    if (i < im.N) {
-        int b;
-        v3<T> ni = ld(xb, i);
-        v3<T> B = local_field(St, xb, i, ni, b);
-        v3<T> Bz = mk(St.Bz[b][0], St.Bz[b][1], St.Bz[b][2]);
-        v3<T> pg = dot(B, ni) * ni - B;  // tangent-space part of dH/dn = -B
-        st(G, im.spin0 + (long long)im.nu * im.N + i, pg);
-        T th = T(0);
-        if (im.nu < im.M - 1) {
-            v3<T> nj = ld(xb + im.N, i);
-            v3<T> c = cross(ni, nj);
-            th = atan2(sqrt(dot(c, c)), dot(ni, nj));
-        }
-        if constexpr (std::is_same<T, float>::value) {
-            f2sum e = exact_dot(ni, B + Bz);
-            r[0] = f2sum{-0.5f * e.hi, -0.5f * e.lo};
-            r[1] = exact_square(th);
-        } else {
-            r[0] = -0.5 * ddot(ni, B + Bz);
-            r[1] = th * th;
-        }
-    }
-    image_reduce<2>(r, 0u, part, vb, im.blk0, im.bpi, cnt + bi.g, scal + kS * bi.g + kE);
+    const long long two_per_sm = 2LL * 152 * kBlock;
+    return spins >= 4 * two_per_sm ? 4 : (spins >= 2 * two_per_sm ? 2 : 1);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_g_field(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                                    const Stencil<T> *__restrict__ S, const rec_t<T> *__restrict__ x,
-                                                    rec_t<T> *__restrict__ G, double *part, unsigned *cnt, double *scal)
-{
-    g_field_body<T>(blockIdx.x, blk, img, S, x, G, part, cnt, scal);
-}
+// Every product and sum of the per-image scalars is written with the
+// non-contracting intrinsics: the same bits in every kernel they are inlined
+// into.
+__device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
 
 // Weights (w+, w-) of the forward and backward differences in the improved
-// tangent (Henkelman and Jonsson 2000) of interior image g, from the image
-// energies of the field pass.
-__device__ __forceinline__ void tangent_weights(const double *scal, int g, double *wp_out, double *wm_out)
+// tangent (Henkelman and Jonsson 2000) of an interior image of energy E0, from
+// its neighbours' energies.
+__device__ __forceinline__ void tangent_weights(double Em, double E0, double Ep, double *wp_out, double *wm_out)
 {
-    double Ep = scal[kS * (g + 1) + kE], E0 = scal[kS * g + kE], Em = scal[kS * (g - 1) + kE];
     double wp, wm;
     if (Ep > E0 && E0 > Em) {
         wp = 1;
@@ -354,94 +416,12 @@ __device__ __forceinline__ void tangent_weights(const double *scal, int g, doubl
     *wm_out = wm;
 }
 
-// LOCALW: the weights are computed here from the energies (persistent
-// kernel) instead of read from the slots k_g_weights filled -- the same
-// function of the same values.
-template <typename T, bool LOCALW, typename R>
-__device__ __forceinline__ void g_tangent_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                               const R *x, const R *G, R *Tau, double *part, unsigned *cnt,
-                                               double *scal)
-{
-    BlkInfo bi = blk[vb];
-    ImgInfo im = img[bi.g];
-    int i = bi.t * kBlock + threadIdx.x;
-    long long p = im.spin0 + (long long)im.nu * im.N + i;
-    bool end = im.nu == 0 || im.nu == im.M - 1;
-    // weights of the forward and backward differences, read (or computed
-    // from the three energies) by every thread: no block barrier
-    T s_wp = T(0), s_wm = T(0);
-    if (!end) {
-        if (LOCALW) {
-            double wp, wm;
-            tangent_weights(scal, bi.g, &wp, &wm);
-            s_wp = (T)wp;
-            s_wm = (T)wm;
-        } else {
-            s_wp = (T)scal[kS * bi.g + kWP];
-            s_wm = (T)scal[kS * bi.g + kWM];
-        }
-    }
-    using A = typename Acc<T>::type;
-    A r[2] = {A{}, A{}};
-    if (i < im.N && end) {
-        // endpoints: one-sided difference to the neighbouring image (only its
-        // slope dE/dr is used, for the interpolated path energy)
-        v3<T> xi = ld(x, p);
-        v3<T> t = im.nu == 0 ? ld(x, p + im.N) - xi : xi - ld(x, p - im.N);
-        t = t - dot(t, xi) * xi;
-        st(Tau, p, t);
-        r[0] = acc_dot(t, t);
-        r[1] = acc_dot(ldc(G, p), t);
-    } else if (i < im.N) {
-        v3<T> xi = ld(x, p), xp = ld(x, p + im.N), xm = ld(x, p - im.N);
-        v3<T> t = axpy(s_wp, xp - xi, s_wm * (xi - xm));
-        t = t - dot(t, xi) * xi;
-        st(Tau, p, t);
-        r[0] = acc_dot(t, t);
-        r[1] = acc_dot(ldc(G, p), t);
-    }
-    image_reduce<2>(r, 0u, part, vb, im.blk0, im.bpi, cnt + bi.g, scal + kS * bi.g + kTT);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_g_tangent(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                                      const rec_t<T> *__restrict__ x, const rec_t<T> *__restrict__ G,
-                                                      rec_t<T> *__restrict__ Tau, double *part, unsigned *cnt,
-                                                      double *scal)
-{
-    g_tangent_body<T, false>(blockIdx.x, blk, img, x, G, Tau, part, cnt, scal);
-}
-
-// Tangent weights of every interior image into its slots; one thread per image.
-__global__ void k_g_weights(const ImgInfo *__restrict__ img, int n_img, double *scal)
-{
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_img) return;
-    ImgInfo im = img[g];
-    if (im.nu == 0 || im.nu == im.M - 1) return;
-    tangent_weights(scal, g, &scal[kS * g + kWP], &scal[kS * g + kWM]);
-}
-
-// Slope dE/dr of image g along its normalised tangent.
-__device__ __forceinline__ double slope_of(const double *scal, int g)
-{
-    double tt = scal[kS * g + kTT];
-    return tt > 0 ? scal[kS * g + kGT] / sqrt(tt) : 0.0;
-}
-
 // Energy-weighted length of the segment from image a to a+1 (reading of the
 // paper's spring modulation: arc length of the curve ((1-w) r, w E(r)) over
 // the geodesic distance h, E(r) the cubic Hermite interpolant of the two
 // images' energies and slopes), by adaptive Simpson with Lyness' criterion
 // and Richardson correction to 1e-13 h, subdivision depth at most 40 (an
 // explicit stack of at most 41 intervals).
-// The per-image scalars below are computed both by one-thread-per-image
-// kernels and inside the persistent kernel; every product and sum is written
-// with the non-contracting intrinsics, so that the two give the same bits
-// whatever fused multiply-adds the compiler would otherwise form.
-__device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
-
 __device__ double seg_integrand(double Ea, double Eb, double da, double db, double h, double w, double s)
 {
     double t = s / h, t2 = dmul(t, t);
@@ -485,130 +465,236 @@ __device__ double seg_length(double Ea, double Eb, double da, double db, double 
     return total;
 }
 
-// Energy-weighted length of segment (g, g+1) from the image slots.
-__device__ __forceinline__ double segment_of(const double *scal, int g, double w)
-{
-    return seg_length(scal[kS * g + kE], scal[kS * (g + 1) + kE], slope_of(scal, g), slope_of(scal, g + 1),
-                      sqrt(scal[kS * g + kL2]), w);
-}
-
-// scal[8g + kLW] = energy-weighted length of segment (g, g+1), one thread per image.
-__global__ void k_g_seglen(const ImgInfo *__restrict__ img, int n_img, double w, double *scal)
-{
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_img) return;
-    ImgInfo im = img[g];
-    if (im.nu >= im.M - 1) return;
-    scal[kS * g + kLW] = segment_of(scal, g, w);
-}
-
-// The force coefficient a of every interior image (F = -Pg + a tau):
-// climbing image (the chain's highest interior image when climbing is on and
-// the image has no fixed kind): a = 2 Pg.tau / |tau|^2; falling image: 0;
-// otherwise (Pg.tau / |tau| + k (l_g - l_{g-1})) / |tau|, l the geodesic or
-// energy-weighted segment lengths.  One thread per image.
-// lw_g, lw_gm: the energy-weighted lengths of segments (g, g+1) and
-// (g-1, g) (used when `weighted`).
-__device__ __forceinline__ double force_coef(const ImgInfo &im, int g, double kspring, int climbing, int weighted,
-                                             const double *scal, double lw_g, double lw_gm)
-{
-    int ci = -1;
-    if (climbing && im.kind < 0) {
-        ci = 1;
-        double best = scal[kS * (im.g0 + 1) + kE];
-        for (int nu = 2; nu < im.M - 1; ++nu) {
-            double e = scal[kS * (im.g0 + nu) + kE];
-            if (e > best) {
-                best = e;
-                ci = nu;
-            }
-        }
-    }
-    double tt = scal[kS * g + kTT];
-    double inv = tt > 0 ? 1.0 / sqrt(tt) : 0.0;
-    double gt = dmul(scal[kS * g + kGT], inv);
-    double fs = weighted ? dmul(kspring, lw_g - lw_gm)
-                         : dmul(kspring, sqrt(scal[kS * g + kL2]) - sqrt(scal[kS * (g - 1) + kL2]));
-    int kind = im.kind >= 0 ? im.kind : (im.nu == ci ? SP_IMAGE_CLIMBING : SP_IMAGE_NORMAL);
-    // climbing: tangential component inverted, no spring; falling: the full
-    // projected gradient, no spring (descends to a minimum along the path)
-    double coef = kind == SP_IMAGE_CLIMBING ? 2.0 * gt : (kind == SP_IMAGE_FALLING ? 0.0 : dadd(gt, fs));
-    return dmul(coef, inv);
-}
-
-__global__ void k_g_coef(const ImgInfo *__restrict__ img, int n_img, double kspring, int climbing, int weighted,
-                         double *scal)
-{
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_img) return;
-    ImgInfo im = img[g];
-    if (im.nu == 0 || im.nu == im.M - 1) return;
-    scal[kS * g + kA] = force_coef(im, g, kspring, climbing, weighted, scal, weighted ? scal[kS * g + kLW] : 0.0,
-                                   weighted ? scal[kS * (g - 1) + kLW] : 0.0);
-}
-
-// Coefficients of the force pass when computed in place (persistent kernel).
 struct CoefArgs {
     double kspring, w;
     int climbing, weighted;
 };
 
-template <typename T, bool LOCALC, typename R>
+// What image nu of a chain does: its own kind, or normal / climbing (ci).
+__device__ __forceinline__ int im_kind(int kind, int nu, int ci)
+{
+    return kind >= 0 ? kind : (nu == ci ? SP_IMAGE_CLIMBING : SP_IMAGE_NORMAL);
+}
+
+// After the field pass: tangents, segment lengths and force coefficients of
+// the chain whose first image is g, by one warp, a lane per image.
+// The force coefficient a of an interior image (F = -Pg + a tau): climbing
+// image (the chain's highest interior image when climbing is on, and the image
+// has no fixed kind): a = 2 Pg.tau / |tau|^2; falling image: 0; otherwise
+// (Pg.tau / |tau| + k (l_g - l_{g-1})) / |tau|, l the geodesic or
+// energy-weighted segment lengths.
+// What bounds it: one trip to memory and the FP64 divisions and square roots
+// of one image (a thread per image whose search for the highest image read the
+// energies one after another took as long, and the tangent weights a launch of
+// 3 us before it).
+template <typename T>
+__device__ void chain_coefs(int g0, const ImgInfo *img, double *scal, CoefArgs ca)
+{
+    const ImgInfo im = img[g0];
+    if (im.nu != 0 || threadIdx.x >= 32) return;
+    const int l = threadIdx.x, M = im.M;
+    // the highest interior image, the first of equals
+    int ci = 1;
+    if (M > 2) {
+        double best = __ldcg(scal + kS * (g0 + 1) + kE);
+        for (int nu = 2 + l; nu < M - 1; nu += 32) {
+            const double e = __ldcg(scal + kS * (g0 + nu) + kE);
+            if (e > best) {
+                best = e;
+                ci = nu;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double e = xor_of(best, o);
+            const int n = __shfl_xor_sync(0xffffffffu, ci, o);
+            if (e > best || (e == best && n < ci)) {
+                best = e;
+                ci = n;
+            }
+        }
+    }
+    if (!ca.climbing) ci = -1;
+    // |tau|^2 and Pg.tau with the weights as the force pass uses them; at the
+    // endpoints one-sided differences (for the slopes)
+    for (int nu = l; nu < M; nu += 32) {
+        double *sc = scal + kS * (g0 + nu);
+        const double *sm = nu > 0 ? sc - kS : sc, *sp = nu < M - 1 ? sc + kS : sc;
+        const double E0 = __ldcg(sc + kE), Em = __ldcg(sm + kE), Ep = __ldcg(sp + kE), L = __ldcg(sc + kL2),
+                     Lm = __ldcg(sm + kL2), pp = __ldcg(sc + kPP), pm = __ldcg(sc + kPM), mm = __ldcg(sc + kMM),
+                     gp = __ldcg(sc + kGP), gm = __ldcg(sc + kGM);
+        double wp = 1.0, wm = 0.0;
+        if (nu == M - 1) {
+            wp = 0.0;
+            wm = 1.0;
+        } else if (nu > 0) {
+            tangent_weights(Em, E0, Ep, &wp, &wm);
+        }
+        wp = (double)(T)wp;
+        wm = (double)(T)wm;
+        const double tt = dadd(dadd(dmul(dmul(wp, wp), pp), dmul(dmul(wm, wm), mm)), dmul(dmul(2.0 * wp, wm), pm));
+        const double gt = dadd(dmul(wp, gp), dmul(wm, gm)), inv = tt > 0 ? 1.0 / sqrt(tt) : 0.0;
+        sc[kWP] = wp;
+        sc[kWM] = wm;
+        sc[kTT] = tt;
+        sc[kGT] = gt;
+        const int kind = im_kind(img[g0 + nu].kind, nu, ci);
+        // climbing: tangential component inverted, no spring; falling: the full
+        // projected gradient, no spring (descends to a minimum along the path)
+        const double gn = dmul(gt, inv);
+        double coef = kind == SP_IMAGE_CLIMBING ? 2.0 * gn : (kind == SP_IMAGE_FALLING ? 0.0 : gn);
+        if (kind == SP_IMAGE_NORMAL && !ca.weighted) coef = dadd(gn, dmul(ca.kspring, sqrt(L) - sqrt(Lm)));
+        sc[kA] = dmul(coef, inv);
+    }
+    if (!ca.weighted) return;
+    // energy-weighted springs: the lengths need the slopes of both ends
+    __threadfence_block();
+    __syncwarp();
+    auto at = [&](int nu, int k) { return *(const volatile double *)(scal + kS * (g0 + nu) + k); };
+    auto slope = [&](int nu) {
+        const double tt = at(nu, kTT);
+        return tt > 0 ? at(nu, kGT) / sqrt(tt) : 0.0;
+    };
+    for (int nu = l; nu < M - 1; nu += 32)
+        scal[kS * (g0 + nu) + kLW] =
+            seg_length(at(nu, kE), at(nu + 1, kE), slope(nu), slope(nu + 1), sqrt(at(nu, kL2)), ca.w);
+    __threadfence_block();
+    __syncwarp();
+    for (int nu = 1 + l; nu < M - 1; nu += 32) {
+        if (im_kind(img[g0 + nu].kind, nu, ci) != SP_IMAGE_NORMAL) continue;
+        const double tt = at(nu, kTT), inv = tt > 0 ? 1.0 / sqrt(tt) : 0.0;
+        const double fs = dmul(ca.kspring, at(nu, kLW) - at(nu - 1, kLW));
+        scal[kS * (g0 + nu) + kA] = dmul(dadd(dmul(at(nu, kGT), inv), fs), inv);
+    }
+}
+template <typename T>
+__global__ void k_g_coefs(const ImgInfo *__restrict__ img, double *scal, const CoefArgs ca)
+{
+    chain_coefs<T>(blockIdx.x, img, scal, ca);
+}
+
+struct NoPost2 {
+    __device__ void operator()(int) const {}
+};
+
+template <typename T, typename R>
+__device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
+                                             const Stencil<T> *__restrict__ S, const R *x, R *G, double *part,
+                                             unsigned *cnt, double *scal)
+{
+    BlkInfo bi = blk[vb];
+    ImgInfo im = img[bi.g];
+    // the chain's stencil, staged in shared memory for the neighbour loop
+    __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
+    Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
+    stage_stencil(S + bi.chain, &St);
+    const long long base = im.spin0 + (long long)im.nu * im.N;
+    const R *xb = x + base;
+    const bool has_p = im.nu < im.M - 1, has_m = im.nu > 0;
+    // every sum in FP64, or float-float for FP32 (the same sums of the same
+    // products to ~1e-14, off the FP64 pipe)
+    using A = typename Acc<T>::type;
+    A r[8] = {};
+    for (int s = 0; s < im.spt; ++s) {
+        const int i = (bi.t * im.spt + s) * kBlock + (int)threadIdx.x;
+        if (i >= im.N) break;
+        int b;
+        const v3<T> ni = ld(xb, i);
+        v3<T> B;
+        if constexpr (std::is_same<T, float>::value) {
+            v3<T> lo;
+            B = local_field_comp(St, xb, i, ni, b, lo);
+            // r[0] collects n.(B + Bz), B = hi + lo; the -1/2 follows at the end
+            acc_add(r[0], ni, B);
+            acc_add(r[0], ni, mk(St.Bz[b][0], St.Bz[b][1], St.Bz[b][2]));
+            r[0].lo += xdot(ni, lo);
+            B = B + lo;
+        } else {
+            B = local_field(St, xb, i, ni, b);
+            r[0] += xdot(ni, B + mk(St.Bz[b][0], St.Bz[b][1], St.Bz[b][2]));
+        }
+        const v3<T> pg = minus_tangent(B, ni);  // tangent-space part of dH/dn = -B
+        st(G, base + i, pg);
+        asm volatile("" ::: "memory");  // the neighbours' registers first, then those of the images
+        const v3<T> np = has_p ? ldc(xb + im.N, i) : ni, nm = has_m ? ldc(xb - im.N, i) : ni;
+        v3<T> dp = np - ni, dm = ni - nm;
+        dp = tangent(dp, ni);
+        dm = tangent(dm, ni);
+        if (has_p) {
+            const v3<T> c = xcross(ni, np);
+            const T th = atan2(sqrt(xdot(c, c)), xdot(ni, np));
+            acc_add(r[1], th, th);
+            acc_add(r[kPP], dp, dp);
+            acc_add(r[kGP], pg, dp);
+        }
+        if (has_m) {
+            acc_add(r[kMM], dm, dm);
+            acc_add(r[kGM], pg, dm);
+        }
+        if (has_p && has_m) acc_add(r[kPM], dp, dm);
+    }
+    if constexpr (std::is_same<T, float>::value)
+        r[0] = f2sum{-0.5f * r[0].hi, -0.5f * r[0].lo};
+    else
+        r[0] *= -0.5;
+    image_sums<8, false>(r, A{}, part, vb, im.blk0, im.bpi, cnt + bi.g, scal + kS * bi.g, NoPost2());
+}
+static_assert(kE == 0 && kL2 == 1 && kGM == 6 && kVF == 7, "the field pass writes slots 0..7 (7: padding)");
+
+template <typename T>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_GF_MINB : 1) k_g_field(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
+                                                    const Stencil<T> *__restrict__ S, const rec_t<T> *__restrict__ x,
+                                                    rec_t<T> *__restrict__ G, double *part, unsigned *cnt, double *scal)
+{
+    g_field_body<T>(blockIdx.x, blk, img, S, x, G, part, cnt, scal);
+}
+
+// mode 0: F only; 1: v from memory (the call's first iteration); 2: v = c F,
+// c the projection coefficient of the previous force pass (read before this
+// block's ticket, so before the image's last block replaces it).
+template <typename T, typename R>
 __device__ __forceinline__ void g_force_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                             R *v, R *F, const R *G, const R *Tau, T dth_m, int mode, double *part,
-                                             unsigned *cnt, double *scal, CoefArgs ca)
+                                             const R *x, const R *v, R *F, const R *G, T dth_m, int mode, double *part,
+                                             unsigned *cnt, double *scal)
 {
     BlkInfo bi = blk[vb];
     ImgInfo im = img[bi.g];
     if (im.nu == 0 || im.nu == im.M - 1) return;
-    // the image's force is -G + a Tau (a from k_g_coef, or computed here from
-    // the same slots by the same function)
-    // (k_g_coef's slot: every thread reads it, no block barrier; computed in
-    // place: thread 0 evaluates it once and the block waits)
-    __shared__ T sh_a;
-    T s_a;
-    if (LOCALC) {
-        if (threadIdx.x == 0) {
-            double lw = 0, lwm = 0;
-            if (ca.weighted) {
-                lw = segment_of(scal, bi.g, ca.w);
-                lwm = segment_of(scal, bi.g - 1, ca.w);
-            }
-            sh_a = (T)force_coef(im, bi.g, ca.kspring, ca.climbing, ca.weighted, scal, lw, lwm);
-        }
-        __syncthreads();
-        s_a = sh_a;
-    } else {
-        s_a = (T)scal[kS * bi.g + kA];
-    }
-    int i = bi.t * kBlock + threadIdx.x;
-    long long p = im.spin0 + (long long)im.nu * im.N + i;
+    double *sc = scal + kS * bi.g;
+    const T a = (T)sc[kA], wp = (T)sc[kWP], wm = (T)sc[kWM], c = mode == 2 ? (T)sc[kC] : T(0);
+    const long long base = im.spin0 + (long long)im.nu * im.N;
     using A = typename Acc<T>::type;
-    A r[3] = {A{}, A{}, A{}};
-    if (i < im.N) {
-        v3<T> Fn = axpy(s_a, ld(Tau, p), -ldc(G, p));
-        if (mode == 1) {
-            v3<T> vi = axpy(dth_m, ldc(F, p) + Fn, ldc(v, p));
-            st(v, p, vi);
-            r[0] = acc_dot(vi, Fn);
+    A r[2] = {}, mx{};
+    for (int s = 0; s < im.spt; ++s) {
+        const int i = (bi.t * im.spt + s) * kBlock + (int)threadIdx.x;
+        if (i >= im.N) break;
+        const long long p = base + i;
+        const v3<T> xi = ld(x, p), xp = ld(x, p + im.N), xm = ld(x, p - im.N);
+        v3<T> t = axpy(wp, xp - xi, wm * (xi - xm));
+        t = tangent(t, xi);
+        const v3<T> Fn = axpy(a, t, -ldc(G, p));
+        if (mode) {
+            const v3<T> Fo = ldc((const R *)F, p);
+            const v3<T> vi = axpy(dth_m, Fo + Fn, mode == 1 ? ldc(v, p) : c * Fo);
+            acc_add(r[0], vi, Fn);
         }
         st(F, p, Fn);
-        r[1] = acc_dot(Fn, Fn);
-        r[2] = r[1];  // max |F|^2; the image's max |F| is its square root
+        const A f2 = acc_dot(Fn, Fn);
+        r[1] = r[1] + f2;
+        mx = nan_max(mx, f2);  // max |F|^2; the image's max |F| is its square root
     }
-    image_reduce<3>(r, 4u, part, vb, im.blk0, im.bpi, cnt + bi.g, scal + kS * bi.g + kVF, ProjectionPost());
+    image_sums<2, true>(r, mx, part, vb, im.blk0, im.bpi, cnt + bi.g, sc + kVF, ForcePost{sc + kVF});
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_g_force(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                                    rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F,
-                                                    const rec_t<T> *__restrict__ G, const rec_t<T> *__restrict__ Tau,
-                                                    T dth_m, int mode, double *part, unsigned *cnt, double *scal)
+                                                    const rec_t<T> *__restrict__ x, const rec_t<T> *__restrict__ v,
+                                                    rec_t<T> *__restrict__ F, const rec_t<T> *__restrict__ G, T dth_m,
+                                                    int mode, double *part, unsigned *cnt, double *scal)
 {
-    g_force_body<T, false>(blockIdx.x, blk, img, v, F, G, Tau, dth_m, mode, part, cnt, scal, CoefArgs{});
+    g_force_body<T>(blockIdx.x, blk, img, x, v, F, G, dth_m, mode, part, cnt, scal);
 }
 
-// mode 0: move; 1: project then move; 2: project only
+// mode 0: move with the stored v; 1: move with v = c F; 2: store v = c F
 template <typename T, typename R>
 __device__ __forceinline__ void g_move_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
                                             R *x, R *v, const R *F, T dt, T dt2_2m, int mode, const double *scal)
@@ -619,17 +705,17 @@ __device__ __forceinline__ void g_move_body(int vb, const BlkInfo *__restrict__ 
     // projection coefficient of the last force pass: every thread reads the
     // image's slot (one broadcast load, no block barrier)
     const T c = mode >= 1 ? (T)scal[kS * bi.g + kC] : T(0);
-    int i = bi.t * kBlock + threadIdx.x;
-    if (i >= im.N) return;
-    long long p = im.spin0 + (long long)im.nu * im.N + i;
-    v3<T> vi;
-    if (mode >= 1) {
-        vi = c * ldc(F, p);
-        st(v, p, vi);
-    } else {
-        vi = ldc(v, p);
+    const long long base = im.spin0 + (long long)im.nu * im.N;
+    for (int s = 0; s < im.spt; ++s) {
+        const int i = (bi.t * im.spt + s) * kBlock + (int)threadIdx.x;
+        if (i >= im.N) break;
+        const long long p = base + i;
+        const v3<T> Fi = ldc(F, p), vi = mode >= 1 ? c * Fi : ldc((const R *)v, p);
+        if (mode == 2)
+            st(v, p, vi);
+        else
+            st(x, p, xunit(axpy(dt2_2m, Fi, axpy(dt, vi, ldc((const R *)x, p)))));
     }
-    if (mode <= 1) st(x, p, normalised(axpy(dt2_2m, ldc(F, p), axpy(dt, vi, ldc(x, p)))));
 }
 
 template <typename T>
@@ -685,22 +771,20 @@ template <typename T> struct PersistArgs {
     const BlkInfo *blk;
     const ImgInfo *img;
     const Stencil<T> *S;
-    rec_t<T> *x, *v, *F, *G, *Tau;
+    rec_t<T> *x, *v, *F, *G;
     double *part, *scal;
     unsigned *cnt;
     T dt, dt2_2m, dth_m;
-    int n_blk, n_iter, first_mode;  // first_mode: move mode of the first iteration (0 or 1)
+    int n_blk, n_img, n_iter;
     CoefArgs ca;
     unsigned *bar, *abort_flag, *status;
     long long limit;
 };
 
-// n_iter GNEB iterations (move, field, tangent, force) of every image of
-// every chain in one cooperative launch: each pass is a grid-stride loop over
-// the block table, the passes are separated by grid barriers, and the
-// per-image tangent weights and force coefficients are computed by each work
-// block from the slots the previous pass filled (the same functions of the
-// same values as the per-pass kernels, so the iterates are bit-identical).
+// n_iter GNEB iterations (move, field, coefs, force) of every image of every chain in
+// one cooperative launch (coefs: a warp per chain): each pass is a grid-stride loop over the block
+// table, the passes are separated by grid barriers.  The bodies are those of
+// the per-pass kernels, so the iterates are bit-identical.
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_g_persistent(const __grid_constant__ PersistArgs<T> a)
 {
@@ -709,12 +793,11 @@ __global__ void __launch_bounds__(kBlock) k_g_persistent(const __grid_constant__
     using R = typename ShRec<T>::type;
     static_assert(sizeof(R) == sizeof(rec_t<T>), "plain-load records have the record layout");
     R *x = reinterpret_cast<R *>(a.x), *v = reinterpret_cast<R *>(a.v), *F = reinterpret_cast<R *>(a.F),
-      *G = reinterpret_cast<R *>(a.G), *Tau = reinterpret_cast<R *>(a.Tau);
+      *G = reinterpret_cast<R *>(a.G);
     unsigned gen = 0;
     for (int it = 0; it < a.n_iter; ++it) {
-        const int mode = it == 0 ? a.first_mode : 1;
         for (int vb = blockIdx.x; vb < a.n_blk; vb += gridDim.x) {
-            g_move_body<T>(vb, a.blk, a.img, x, v, (const R *)F, a.dt, a.dt2_2m, mode, a.scal);
+            g_move_body<T>(vb, a.blk, a.img, x, v, (const R *)F, a.dt, a.dt2_2m, it ? 1 : 0, a.scal);
             __syncthreads();
         }
         if (!grid_sync(a.bar, a.abort_flag, gen, a.limit, a.status, 1u)) return;
@@ -723,14 +806,11 @@ __global__ void __launch_bounds__(kBlock) k_g_persistent(const __grid_constant__
             __syncthreads();
         }
         if (!grid_sync(a.bar, a.abort_flag, gen, a.limit, a.status, 1u)) return;
-        for (int vb = blockIdx.x; vb < a.n_blk; vb += gridDim.x) {
-            g_tangent_body<T, true>(vb, a.blk, a.img, (const R *)x, (const R *)G, Tau, a.part, a.cnt, a.scal);
-            __syncthreads();
-        }
+        for (int g = blockIdx.x; g < a.n_img; g += gridDim.x) chain_coefs<T>(g, a.img, a.scal, a.ca);
         if (!grid_sync(a.bar, a.abort_flag, gen, a.limit, a.status, 1u)) return;
         for (int vb = blockIdx.x; vb < a.n_blk; vb += gridDim.x) {
-            g_force_body<T, true>(vb, a.blk, a.img, v, F, (const R *)G, (const R *)Tau, a.dth_m, 1, a.part, a.cnt,
-                                  a.scal, a.ca);
+            g_force_body<T>(vb, a.blk, a.img, (const R *)x, (const R *)v, F, (const R *)G, a.dth_m, it ? 2 : 1, a.part,
+                            a.cnt, a.scal);
             __syncthreads();
         }
         if (!grid_sync(a.bar, a.abort_flag, gen, a.limit, a.status, 1u)) return;
@@ -764,8 +844,8 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
     MinScratch *s = *sp;
     int N = S.N;
     int nblk = blocks_for(N > 0 ? N : 1);
-    if (grow(s->F, sizeof(rec_t<T>) * (size_t)(N > 0 ? N : 1)) || grow(s->scal, 8 * sizeof(double)) ||
-        grow(s->part, 3 * sizeof(double) * (size_t)nblk) || grow_counters(s->cnt, 1, st) ||
+    if (grow(s->F, sizeof(rec_t<T>) * (size_t)(N > 0 ? N : 1)) || grow(s->scal, kS * sizeof(double)) ||
+        grow(s->part, kPartRow * sizeof(double) * (size_t)nblk) || grow_counters(s->cnt, 1, st) ||
         grow(s->state, 4 * sizeof(int)))
         return SP_ERR_CUDA;
     rec_t<T> *x = (rec_t<T> *)n, *vv = (rec_t<T> *)v, *F = (rec_t<T> *)s->F.p;
@@ -774,14 +854,16 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
     int *state = (int *)s->state.p;
     double dth_m = a.dt / (2.0 * a.mass), dt2_2m = a.dt * a.dt / (2.0 * a.mass);
     if (cudaMemsetAsync(state, 0, 4 * sizeof(int), st) != cudaSuccess) return SP_ERR_CUDA;
-    launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, x, vv, F, (T)dth_m, 0, part, cnt, scal, (const int *)state);
+    launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F, (T)dth_m, 0, part, cnt,
+               scal, (const int *)state);
     int k = 0;
     while (k < a.max_iter) {
         int chunk = std::min(a.check_every, a.max_iter - k);
         for (int c = 0; c < chunk; ++c, ++k) {
             launch_pdl(k_vp_move<T>, dim3(nblk), dim3(kBlock), 0, st, N, x, vv, (const rec_t<T> *)F, (T)a.dt, (T)dt2_2m, a.tol, k,
                        a.max_iter, (const double *)scal, state);
-            launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, x, vv, F, (T)dth_m, 1, part, cnt, scal, (const int *)state);
+            launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F, (T)dth_m,
+                       k == 0 ? 1 : 2, part, cnt, scal, (const int *)state);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
         if (cudaMemcpyAsync(s->host_state, state, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -793,7 +875,7 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
     launch_pdl(k_vp_move<T>, dim3(nblk), dim3(kBlock), 0, st, N, x, vv, (const rec_t<T> *)F, (T)a.dt, (T)dt2_2m, a.tol,
                a.max_iter, a.max_iter, (const double *)scal, state);
     if (cudaMemcpyAsync(s->host_state, state, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(s->host_fmax, scal + 2, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(s->host_fmax, scal + kFMAX, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return SP_ERR_CUDA;
     *iters = s->host_state[0];
@@ -802,41 +884,34 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
 }
 
 // ------------------------------------------------------------ batched VP
-// One image per system.  Per system g: scal[8g + kVF, kFF, kFMAX] from the
-// last force pass, state[2g] iterations moved, state[2g+1] active flag,
-// proj[g] whether the last force pass updated the velocity.
+// One image per system.  Per system g: the slots kVF.. from the last force
+// pass, state[2g] iterations moved, state[2g+1] active flag, proj[g] whether
+// the last force pass had a velocity.
+// 1 M spins in 64 systems: 56 -> 52 us an iteration; bound by the chain of a
+// block (tables, state, neighbours, block sum, ticket) with 6 blocks per SM
+// in flight (5: 53, 4: 56).
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_bvp_force(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_bvp_force(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
                                                       const Stencil<T> *__restrict__ S, const rec_t<T> *__restrict__ x,
-                                                      rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
+                                                      const rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
                                                       int mode, double *part, unsigned *cnt, double *scal,
                                                       const int *state, int *proj)
 {
+    // the tables and stencils do not change while kernels are in flight
+    const BlkInfo bi = blk[blockIdx.x];
+    const ImgInfo im = img[bi.g];
+    __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
+    Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
+    stage_stencil(S + bi.chain, &St);
     allow_dependents();
     wait_prerequisite();  // state, scalars and records come from the kernels before
-    BlkInfo bi = blk[blockIdx.x];
-    ImgInfo im = img[bi.g];
-    if (mode == 1 && state[2 * bi.g + 1] == 0) return;
-    const Stencil<T> &St = S[im.chain];
-    int i = bi.t * kBlock + threadIdx.x;
-    const rec_t<T> *xb = x + im.spin0;
-    T r[3] = {0, 0, 0};
-    if (i < im.N) {
-        int b;
-        long long p = im.spin0 + i;
-        v3<T> ni = ld(xb, i);
-        v3<T> B = local_field(St, xb, i, ni, b);
-        v3<T> Fn = B - dot(B, ni) * ni;
-        if (mode == 1) {
-            v3<T> vi = axpy(dth_m, ldc(F, p) + Fn, ldc(v, p));
-            st(v, p, vi);
-            r[0] = dot(vi, Fn);
-        }
-        st(F, p, Fn);
-        r[1] = dot(Fn, Fn);
-        r[2] = r[1];
-    }
-    image_reduce<3>(r, 4u, part, blockIdx.x, im.blk0, im.bpi, cnt + bi.g, scal + kS * bi.g + kVF, ProjectionPost());
+    if (mode && state[2 * bi.g + 1] == 0) return;
+    double *sc = scal + kS * bi.g;
+    const T c = mode == 2 ? (T)sc[kC] : T(0);
+    const int i = bi.t * kBlock + threadIdx.x;
+    T r[2] = {0, 0}, mx = 0;
+    if (i < im.N) vp_force(St, x + im.spin0, v + im.spin0, F + im.spin0, i, dth_m, mode, c, r, mx);
+    image_sums<2, true>(r, mx, part, blockIdx.x, im.blk0, im.bpi, cnt + bi.g, sc + kVF, ForcePost{sc + kVF});
     if (bi.t == 0 && threadIdx.x == 0) proj[bi.g] = mode;
 }
 
@@ -847,32 +922,16 @@ __global__ void __launch_bounds__(kBlock) k_bvp_move(const BlkInfo *__restrict__
                                                      int k, int max_iter, const double *scal, int *state,
                                                      const int *proj)
 {
+    const BlkInfo bi = blk[blockIdx.x];
+    const ImgInfo im = img[bi.g];
     allow_dependents();
     wait_prerequisite();  // state, scalars and records come from the kernels before
-    BlkInfo bi = blk[blockIdx.x];
-    ImgInfo im = img[bi.g];
     const double *sc = scal + kS * bi.g;
-    __shared__ T s_c;
-    __shared__ int s_done;
-    if (threadIdx.x == 0) {
-        s_c = (T)sc[kC];
-        s_done = (sqrt(sc[kFMAX]) < tol) || (k >= max_iter);
-    }
-    __syncthreads();
-    bool done = s_done;
-    int i = bi.t * kBlock + threadIdx.x;
-    if (i < im.N) {
-        long long p = im.spin0 + i;
-        v3<T> vi;
-        if (proj[bi.g]) {
-            T c = s_c;
-            vi = c * ldc(F, p);
-            st(v, p, vi);
-        } else {
-            vi = ldc(v, p);
-        }
-        if (!done) st(x, p, normalised(axpy(dt2_2m, ldc(F, p), axpy(dt, vi, ldc(x, p)))));
-    }
+    const bool done = sc[kFN] < tol || k >= max_iter;
+    const int i = bi.t * kBlock + threadIdx.x;
+    if (i < im.N)
+        vp_move(x + im.spin0, v + im.spin0, F + im.spin0, i, dt, dt2_2m, proj[bi.g] != 0, (T)sc[kC], done,
+                k >= max_iter);
     if (bi.t == 0 && threadIdx.x == 0) {
         state[2 * bi.g + 1] = done ? 0 : 1;
         if (!done) state[2 * bi.g] = k + 1;
@@ -893,15 +952,15 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
     for (int c = 0; c < C; ++c) {
         int N = stencils[c].N;
         int bpi = blocks_for(N > 0 ? N : 1);
-        ImgInfo im{spin0[c], N, c, 0, 1, c, (int)blk.size(), bpi, -1};
-        for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{c, t});
+        ImgInfo im{spin0[c], N, c, 0, 1, c, (int)blk.size(), bpi, -1, 1};
+        for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{c, t, c});
         img.push_back(im);
         total = std::max(total, spin0[c] + (long long)N);
     }
     int n_full = (int)blk.size();
     size_t rb = sizeof(rec_t<T>) * (size_t)std::max(total, 1LL);
     // blk holds the full table followed by room for a compacted copy
-    if (grow(s->F, rb) || grow(s->scal, kS * sizeof(double) * C) || grow(s->part, 3 * sizeof(double) * (size_t)n_full) ||
+    if (grow(s->F, rb) || grow(s->scal, kS * sizeof(double) * C) || grow(s->part, kPartRow * sizeof(double) * (size_t)n_full) ||
         grow_counters(s->cnt, C, st) || grow(s->blk, 2 * sizeof(BlkInfo) * n_full) ||
         grow(s->img, sizeof(ImgInfo) * C) || grow(s->sten, sizeof(Stencil<T>) * C) ||
         grow(s->state, sizeof(int) * 3 * C))
@@ -924,7 +983,7 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
     double dth_m = a.dt / (2.0 * a.mass), dt2_2m = a.dt * a.dt / (2.0 * a.mass);
     std::vector<int> hs(2 * C);
     launch_pdl(k_bvp_force<T>, dim3(n_full), dim3(kBlock), 0, st, (const BlkInfo *)Bfull, (const ImgInfo *)I, Sd,
-               (const rec_t<T> *)x, v, F, (T)dth_m, 0, part, cnt, scal, (const int *)state, proj);
+               (const rec_t<T> *)x, (const rec_t<T> *)v, F, (T)dth_m, 0, part, cnt, scal, (const int *)state, proj);
     int k = 0, n_act = n_full;
     while (k < a.max_iter) {
         int chunk = std::min(a.check_every, a.max_iter - k);
@@ -933,7 +992,8 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
                        (const rec_t<T> *)F, (T)a.dt, (T)dt2_2m, a.tol, k, a.max_iter, (const double *)scal, state,
                        (const int *)proj);
             launch_pdl(k_bvp_force<T>, dim3(n_act), dim3(kBlock), 0, st, (const BlkInfo *)Bact, (const ImgInfo *)I, Sd,
-                       (const rec_t<T> *)x, v, F, (T)dth_m, 1, part, cnt, scal, (const int *)state, proj);
+                       (const rec_t<T> *)x, (const rec_t<T> *)v, F, (T)dth_m, k == 0 ? 1 : 2, part, cnt, scal,
+                       (const int *)state, proj);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
         if (cudaMemcpyAsync(hs.data(), state, sizeof(int) * 2 * C, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -947,7 +1007,7 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
         for (int c = 0; c < C; ++c)
             if (hs[2 * c + 1]) {
                 img[c].blk0 = (int)act.size();
-                for (int t = 0; t < img[c].bpi; ++t) act.push_back(BlkInfo{c, t});
+                for (int t = 0; t < img[c].bpi; ++t) act.push_back(BlkInfo{c, t, c});
             }
         if (act.empty()) break;
         if (4 * (long long)act.size() <= 3LL * n_act) {
@@ -989,20 +1049,21 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
     long long total = 0;
     for (int c = 0; c < C; ++c) {
         int N = stencils[c].N;
-        int bpi = blocks_for(N > 0 ? N : 1);
+        const int spt = gneb_spt((long long)M[c] * N);
+        int bpi = blocks_for(N > 0 ? N : 1, kBlock * spt);
         int g0 = (int)img.size();
         for (int nu = 0; nu < M[c]; ++nu) {
             int kind = a.kinds ? a.kinds[g0 + nu] : -1;
-            ImgInfo im{spin0[c], N, c, nu, M[c], g0, (int)blk.size(), bpi, kind};
-            for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{(int)img.size(), t});
+            ImgInfo im{spin0[c], N, c, nu, M[c], g0, (int)blk.size(), bpi, kind, spt};
+            for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{(int)img.size(), t, c});
             img.push_back(im);
         }
         total = std::max(total, spin0[c] + (long long)M[c] * N);
     }
     int n_img = (int)img.size(), n_blk = (int)blk.size();
     size_t rb = sizeof(rec_t<T>) * (size_t)std::max(total, 1LL);
-    if (grow(s->F, rb) || grow(s->G, rb) || grow(s->Tau, rb) || grow(s->scal, kS * sizeof(double) * n_img) ||
-        grow(s->part, 3 * sizeof(double) * (size_t)n_blk) || grow_counters(s->cnt, n_img, st) ||
+    if (grow(s->F, rb) || grow(s->G, rb) || grow(s->scal, kS * sizeof(double) * n_img) ||
+        grow(s->part, kPartRow * sizeof(double) * (size_t)n_blk) || grow_counters(s->cnt, n_img, st) ||
         grow(s->blk, sizeof(BlkInfo) * n_blk) || grow(s->img, sizeof(ImgInfo) * n_img) ||
         grow(s->sten, sizeof(Stencil<T>) * C))
         return SP_ERR_CUDA;
@@ -1026,23 +1087,19 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
     const ImgInfo *I = (const ImgInfo *)s->img.p;
     const Stencil<T> *Sd = (const Stencil<T> *)s->sten.p;
     rec_t<T> *x = (rec_t<T> *)chain, *v = (rec_t<T> *)vel;
-    rec_t<T> *F = (rec_t<T> *)s->F.p, *G = (rec_t<T> *)s->G.p, *Tau = (rec_t<T> *)s->Tau.p;
+    rec_t<T> *F = (rec_t<T> *)s->F.p, *G = (rec_t<T> *)s->G.p;
     double *scal = (double *)s->scal.p, *part = (double *)s->part.p;
     unsigned *cnt = (unsigned *)s->cnt.p;
     double dth_m = a.dt / (2.0 * a.mass), dt2_2m = a.dt * a.dt / (2.0 * a.mass);
-    const int weighted = a.w != 0.0;
-    const int ib = (n_img + 127) / 128;
+    const CoefArgs ca{a.k, a.w, a.climbing, a.w != 0.0};
     auto forces = [&](int mode, cudaStream_t ss) {
         k_g_field<T><<<n_blk, kBlock, 0, ss>>>(B, I, Sd, x, G, part, cnt, scal);
-        k_g_weights<<<ib, 128, 0, ss>>>(I, n_img, scal);
-        k_g_tangent<T><<<n_blk, kBlock, 0, ss>>>(B, I, x, G, Tau, part, cnt, scal);
-        if (weighted) k_g_seglen<<<ib, 128, 0, ss>>>(I, n_img, a.w, scal);
-        k_g_coef<<<ib, 128, 0, ss>>>(I, n_img, a.k, a.climbing, weighted, scal);
-        k_g_force<T><<<n_blk, kBlock, 0, ss>>>(B, I, v, F, G, Tau, dth_m, mode, part, cnt, scal);
+        k_g_coefs<T><<<n_img, 32, 0, ss>>>(I, scal, ca);
+        k_g_force<T><<<n_blk, kBlock, 0, ss>>>(B, I, x, v, F, G, dth_m, mode, part, cnt, scal);
     };
     auto iteration = [&](cudaStream_t ss) {
         k_g_move<T><<<n_blk, kBlock, 0, ss>>>(B, I, x, v, F, a.dt, dt2_2m, 1, scal);
-        forces(1, ss);
+        forces(2, ss);
     };
     forces(0, st);
     int remaining = a.n_iter;
@@ -1058,8 +1115,8 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
             per_sm < 1)
             return SP_ERR_CUDA;
         int grid = (int)std::min<long long>((long long)nsm * per_sm, n_blk);
-        PersistArgs<T> pa{B, I, Sd, x, v, F, G, Tau, part, scal, cnt, (T)a.dt, (T)dt2_2m, (T)dth_m, n_blk, remaining,
-                          0, CoefArgs{a.k, a.w, a.climbing, weighted}, (unsigned *)s->sync.p,
+        PersistArgs<T> pa{B, I, Sd, x, v, F, G, part, scal, cnt, (T)a.dt, (T)dt2_2m, (T)dth_m, n_blk, n_img, remaining,
+                          ca, (unsigned *)s->sync.p,
                           (unsigned *)s->sync.p + 1, a.status, a.wait_limit > 0 ? a.wait_limit : (1LL << 21)};
         void *args[] = {&pa};
         if (cudaMemsetAsync(s->sync.p, 0, 4 * sizeof(unsigned), st) != cudaSuccess ||
@@ -1087,10 +1144,10 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
                 return SP_ERR_CUDA;
         }
         struct GKey {
-            const void *x, *v, *F, *G, *Tau, *scal, *part, *cnt, *blk, *img, *sten;
+            const void *x, *v, *F, *G, *scal, *part, *cnt, *blk, *img, *sten;
             double dt, mass, k, w;
             int climbing, n_blk;
-        } gk{x, v, F, G, Tau, scal, part, cnt, B, I, Sd, a.dt, a.mass, a.k, a.w, a.climbing, n_blk};
+        } gk{x, v, F, G, scal, part, cnt, B, I, Sd, a.dt, a.mass, a.k, a.w, a.climbing, n_blk};
         std::vector<char> gkey(sizeof gk + s->layout.size());
         memcpy(gkey.data(), &gk, sizeof gk);
         memcpy(gkey.data() + sizeof gk, s->layout.data(), s->layout.size());
