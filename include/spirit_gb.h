@@ -647,13 +647,16 @@ enum {
     /* the same for the corrector pass alone */
     SP_OPT_CUBIC_ROWS_CORR = 12,
     /* 1 (default): FP32 stochastic Heun on the 27-point path takes the lean
-     * passes where the lattice's xy plane is cut into whole column tiles of
-     * the tile height in use (nx a multiple of 32; ny of 8 with one column
-     * per thread, of 16 with two); the same method and stencil, fewer
-     * instructions per spin, results equal to the general passes within FP32
-     * rounding (not bit for bit; one and two columns give the same bits).
+     * passes (without the dipole term; one lattice or a batch of replicas); the
+     * same method and stencil, fewer instructions per spin, results equal to the
+     * general passes within FP32 rounding (not bit for bit; one and two columns
+     * give the same bits).  Where neither SP_OPT_CUBIC_ROWS nor a split is set a
+     * single lattice takes two columns per thread in the predictor, and in the
+     * corrector where they make whole tiles.
      * 0: always the general passes.  Reading returns 1 when the lean passes
-     * would be taken for a Heun call of this context */
+     * would be taken for a Heun call of this context and its xy plane is cut
+     * into whole column tiles of the tile height in SP_OPT_CUBIC_ROWS (nx a
+     * multiple of 32; ny of 8 with one column per thread, of 16 with two) */
     SP_OPT_CUBIC_LEAN = 13
 };
 int sp_set_option(sp_ctx *ctx, int option, int value);

@@ -280,6 +280,7 @@ void detect_cubic(sp_ctx *c)
     fill_cubic(c, J, D, Jc, c->Cd);
     c->zc_auto = 0;  // recomputed for the new lattice on first use
     c->zc_auto_corr = 0;
+    c->zc_gen[0] = c->zc_gen[1] = 0;
     c->cubic = true;
 }
 
@@ -377,7 +378,8 @@ template <typename T> int llg_run(sp_ctx *c, void *n, const sp_llg_params *p, in
                (p->solver == SP_HEUN || p->solver == SP_DEPONDT || p->solver == SP_SIB ||
                 (p->solver == SP_RK4 && c->h.dipole == SP_DIPOLE_NONE));
     LlgConst<T> k = llg_const<T>(c, p);
-    int per0 = cub ? cubic_per(c) : 0, per1 = cub ? cubic_per(c, 1) : 0;
+    const bool lean = cub && p->solver == SP_HEUN && cubic_lean_taken(c);
+    int per0 = cub ? cubic_per(c, 0, lean) : 0, per1 = cub ? cubic_per(c, 1, lean) : 0;
     if (c->use_small && c->N <= kSmallMax && c->h.dipole == SP_DIPOLE_NONE && !rk4 && !c->prof.on) {
         if (std::is_same<T, float>::value) {
             // whole steps inside one CTA (the lattice fits in shared memory)
@@ -411,14 +413,14 @@ template <typename T> int llg_run(sp_ctx *c, void *n, const sp_llg_params *p, in
         if ((rc = dipole(c, nn, &bd, st))) return rc;
         int pr = c->prof.begin(SP_PROF_LLG_PREDICTOR, st);
         cudaError_t e = cub ? launch_cubic<T>(0, p->solver, CP, nn, np, q, nn, (const rec_t<T> *)bd, k, per0, st,
-                                              cubic_rows(c, 0), cubic_lean_taken(c, 0))
+                                              cubic_rows(c, 0, lean), lean)
                             : launch_llg_pred<T>(p->solver, S, nn, (const rec_t<T> *)bd, np, q, k, st);
         c->prof.end(pr, st);
         if (e != cudaSuccess) return cuda_fail(c, e, "LLG predictor launch");
         if ((rc = dipole(c, np, &bd, st))) return rc;
         pr = c->prof.begin(SP_PROF_LLG_CORRECTOR, st);
         e = cub ? launch_cubic<T>(1, p->solver, CP, np, nullptr, q, nn, (const rec_t<T> *)bd, k, per1, st,
-                                  cubic_rows(c, 1), cubic_lean_taken(c, 1))
+                                  cubic_rows(c, 1, lean), lean)
                 : launch_llg_corr<T>(p->solver, S, nn, np, q, (const rec_t<T> *)bd, k, st);
         c->prof.end(pr, st);
         if (e != cudaSuccess) return cuda_fail(c, e, "LLG corrector launch");
@@ -501,10 +503,18 @@ int replicas_run(sp_ctx *c, void *n, const sp_llg_params *p, int n_steps, cudaSt
     for (int r = 0; r < n_rep; ++r) hot = hot || temps[r] > 0;
     k.thermal = (hot && p->alpha > 0) ? 1 : 0;
     bool cub = c->cubic && c->use_cubic;  // all four solvers (a batch has no dipole term)
-    int per0 = cub ? cubic_per_batch(c, 0, n_rep) : 0, per1 = cub ? cubic_per_batch(c, 1, n_rep) : 0;
+    const bool lean = cub && p->solver == SP_HEUN && cubic_lean_taken(c);
+    int per0 = cub ? cubic_per_batch(c, 0, n_rep, lean) : 0, per1 = cub ? cubic_per_batch(c, 1, n_rep, lean) : 0;
     // runs of a few planes per CTA are mostly the ring's prologue: the
-    // per-spin kernels are faster there (unless the user fixed the split)
-    if (cub && c->zc == 0 && per0 < kCubicMinRun) cub = false;
+    // per-spin kernels are faster there (unless the user fixed the split).
+    // The lean passes: 32 steps take about 240 + 0.148 U us for U (32 x 8 tile,
+    // plane) units, the per-spin kernels 140 + 1.04 K us for K thousand spins
+    // (29 replicas of 30^3: 723 and 950 us; 12: 439 and 480; 7: 332 and 320; 29
+    // of 24^3: 514 and 562, of 22^3: 617 and 467, of 16^3: 343 and 260)
+    if (cub && c->zc == 0) {
+        const double units = (double)cubic_units(c->nc[0], c->nc[1], c->nc[2]) * n_rep, kspins = 1e-3 * (double)NR;
+        if (lean ? 1.04 * kspins < 100.0 + 0.148 * units : per0 < kCubicMinRun) cub = false;
+    }
     auto one_step = [&](const LlgConst<T> &kk, cudaStream_t s) -> cudaError_t {
         if (rk4) {
             const rec_t<T> *src[4] = {nn, np, q, np};
@@ -516,10 +526,10 @@ int replicas_run(sp_ctx *c, void *n, const sp_llg_params *p, int n_steps, cudaSt
             }
             return cudaSuccess;
         }
-        cudaError_t e = cub ? launch_cubic<T>(0, p->solver, CP, nn, np, q, nn, nullptr, kk, per0, s)
+        cudaError_t e = cub ? launch_cubic<T>(0, p->solver, CP, nn, np, q, nn, nullptr, kk, per0, s, 1, lean)
                             : launch_llg_pred<T>(p->solver, S, nn, nullptr, np, q, kk, s);
         if (e != cudaSuccess) return e;
-        return cub ? launch_cubic<T>(1, p->solver, CP, np, nullptr, q, nn, nullptr, kk, per1, s)
+        return cub ? launch_cubic<T>(1, p->solver, CP, np, nullptr, q, nn, nullptr, kk, per1, s, 1, lean)
                    : launch_llg_corr<T>(p->solver, S, nn, np, q, nullptr, kk, s);
     };
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -535,7 +545,7 @@ int replicas_run(sp_ctx *c, void *n, const sp_llg_params *p, int n_steps, cudaSt
         kk.step_base = ctr;
         struct Key {
             const void *n, *pred, *ctr;
-            int n_rep, solver, cub, per0, per1, G;
+            int n_rep, solver, cub, lean, per0, per1, G;
         } key;
         std::memset(&key, 0, sizeof key);
         key.n = nn;
@@ -544,6 +554,7 @@ int replicas_run(sp_ctx *c, void *n, const sp_llg_params *p, int n_steps, cudaSt
         key.n_rep = n_rep;
         key.solver = p->solver;
         key.cub = cub;
+        key.lean = lean;
         key.per0 = per0;
         key.per1 = per1;
         key.G = G;
@@ -691,11 +702,13 @@ template <typename T> int autotune_run(sp_ctx *c, const void *n, int *chosen, cu
     auto launch = [&](int pass, int per, int rows) {
         return pass == 0
                    ? launch_cubic<T>(0, SP_HEUN, CP, (const rec_t<T> *)n, np, q, nullptr, nullptr, k, per, st, rows,
-                                     cubic_lean_taken(c, 0))
+                                     cubic_lean_taken(c))
                    : launch_cubic<T>(1, SP_HEUN, CP, np, nullptr, q, out, nullptr, k, per, st, rows,
-                                     cubic_lean_taken(c, 1));
+                                     cubic_lean_taken(c));
     };
     int user = c->zc, user_corr = c->zc_corr, user_rows[2] = {c->rows[0], c->rows[1]};
+    const bool user_set[2] = {c->rows_set[0], c->rows_set[1]};
+    c->rows_set[0] = c->rows_set[1] = true;
     c->zc = 0;
     c->zc_corr = 0;
     int best_of[2] = {1, 1}, best_rows[2] = {1, 1};
@@ -708,12 +721,12 @@ template <typename T> int autotune_run(sp_ctx *c, const void *n, int *chosen, cu
         for (int rows = 1; rows <= 2 && e == cudaSuccess; ++rows) {
             c->rows[pass] = rows;
             if (cubic_rows(c, pass) != rows) continue;
-            (pass == 0 ? c->zc_auto : c->zc_auto_corr) = 0;
-            int bal = cubic_per(c, pass);
+            (pass == 0 ? c->zc_auto : c->zc_auto_corr) = c->zc_gen[pass] = 0;
+            int bal = cubic_per(c, pass, cubic_lean_taken(c));
             std::vector<int> cands = {bal, (bal + 1) / 2, (bal + 2) / 3, (bal + 3) / 4, (bal + 5) / 6, 4, 8, 16, 32};
             std::sort(cands.begin(), cands.end());
             cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
-            if (pass == 1) e = launch(0, cubic_per(c, 0), cubic_rows(c, 0));  // the corrector reads its output
+            if (pass == 1) e = launch(0, cubic_per(c, 0, cubic_lean_taken(c)), c->rows[0]);  // the corrector reads its output
             if (rows == 1) best_of[pass] = bal;
             for (int per : cands) {
                 if (per < 1 || e != cudaSuccess) continue;
@@ -739,7 +752,7 @@ template <typename T> int autotune_run(sp_ctx *c, const void *n, int *chosen, cu
             }
         }
         c->rows[pass] = best_rows[pass];
-        (pass == 0 ? c->zc_auto : c->zc_auto_corr) = 0;
+        (pass == 0 ? c->zc_auto : c->zc_auto_corr) = c->zc_gen[pass] = 0;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -748,7 +761,9 @@ template <typename T> int autotune_run(sp_ctx *c, const void *n, int *chosen, cu
         c->zc_corr = user_corr;
         c->rows[0] = user_rows[0];
         c->rows[1] = user_rows[1];
-        c->zc_auto = c->zc_auto_corr = 0;
+        c->rows_set[0] = user_set[0];
+        c->rows_set[1] = user_set[1];
+        c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return cuda_fail(c, e, "autotune");
     }
     c->zc = best_of[0];
@@ -1435,10 +1450,12 @@ int sp_set_option(sp_ctx *c, int option, int value)
         if (value < 0) return fail(c, SP_ERR_ARG, "units per CTA must be >= 0 (0: balanced)");
         c->zc = value;
         c->zc_corr = 0;  // the user's value applies to both passes
+        c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return SP_OK;
     case SP_OPT_PLANES_PER_CTA_CORR:
         if (value < 0) return fail(c, SP_ERR_ARG, "units per CTA must be >= 0 (0: as the predictor)");
         c->zc_corr = value;
+        c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return SP_OK;
     case SP_OPT_MC_RESIDENT:
         if (value != 0 && value != 1) return fail(c, SP_ERR_ARG, "mc_resident takes 0 or 1");
@@ -1449,12 +1466,13 @@ int sp_set_option(sp_ctx *c, int option, int value)
         if (value != 1 && value != 2) return fail(c, SP_ERR_ARG, "columns per thread: 1 or 2");
         if (option == SP_OPT_CUBIC_ROWS) c->rows[0] = value;
         c->rows[1] = value;
-        c->zc_auto = c->zc_auto_corr = 0;
+        c->rows_set[option == SP_OPT_CUBIC_ROWS ? 0 : 1] = true;
+        c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return SP_OK;
     case SP_OPT_CUBIC_LEAN:
         if (value != 0 && value != 1) return fail(c, SP_ERR_ARG, "cubic_lean takes 0 or 1");
         c->lean = value;
-        c->zc_auto = c->zc_auto_corr = 0;
+        c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return SP_OK;
     case SP_OPT_GNEB_PERSISTENT:
         if (value != 0 && value != 1) return fail(c, SP_ERR_ARG, "gneb_persistent takes 0 or 1");
@@ -1517,7 +1535,7 @@ int sp_get_option(const sp_ctx *c, int option, int *value)
         *value = cubic_rows(c, 1);
         return SP_OK;
     case SP_OPT_CUBIC_LEAN:
-        *value = cubic_lean_taken(c, 0) ? 1 : 0;
+        *value = cubic_lean_taken(c) && cubic_lean_fits(c->nc[0], c->nc[1], cubic_rows(c, 0)) ? 1 : 0;  // whole tiles
         return SP_OK;
     case SP_OPT_WAIT_LIMIT:
         *value = c->wait_limit;

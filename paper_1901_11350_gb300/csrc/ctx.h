@@ -127,6 +127,8 @@ struct sp_ctx {
     int zc_corr = 0;        // the corrector's, when the autotuner chose it separately
     int zc_auto = 0;        // balanced value, computed on first use
     int zc_auto_corr = 0;   // the same for the corrector pass (its own occupancy)
+    int zc_gen[2] = {0, 0};  // balanced values of the general passes where Heun takes the lean ones
+    bool rows_set[2] = {false, false};  // rows[] is a choice (option, autotuner)
     int rows[2] = {1, 1};   // columns per thread of the 27-point predictor and corrector (1 or 2)
     int lean = 1;           // the lean FP32 Heun passes where the lattice fits them (SP_OPT_CUBIC_LEAN)
     CubicParams<float> Cf = {};
@@ -175,50 +177,72 @@ int status_enter(sp_ctx *c);
 int status_check_records(sp_ctx *c, const void *recs, long n_rec, unsigned site, cudaStream_t st);
 int status_check_doubles(sp_ctx *c, const double *v, long n_val, unsigned site, cudaStream_t st);
 
-// Units per CTA of the 27-point path for a batch of n_rep replicas: the
-// user's choice, or all replicas' units spread over one wave of resident CTAs.
-inline int cubic_per_batch(sp_ctx *c, int pass, int n_rep)
-{
-    if (pass == 1 && c->zc_corr > 0) return c->zc_corr;
-    if (c->zc > 0) return c->zc;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 1;
-    long slots = (long)nsm * cubic_resident_ctas(c->prec, pass);
-    long units = cubic_units(c->nc[0], c->nc[1], c->nc[2]) * n_rep;
-    return (int)std::max(1L, (units + slots - 1) / slots);
-}
-
-// Columns per thread the 27-point pass of a single lattice takes.
+// Columns per thread the general 27-point pass of a single lattice takes.
 inline int cubic_rows(const sp_ctx *c, int pass)
 {
     return cubic_rows_taken(c->prec, c->rows[pass], false, c->h.dipole != SP_DIPOLE_NONE);
 }
 
 // Whether a Heun pass of this context on the 27-point path takes the lean
-// FP32 kernels (cubic_lean.cu): option on, FP32, no dipole field and a
-// lattice cut into whole column tiles of the pass's height (32 x 8 rows).
-inline bool cubic_lean_taken(const sp_ctx *c, int pass)
+// FP32 kernels (cubic_lean.cu): option on, FP32 and no dipole field.  (Ragged
+// lattices too: the tiles are those of the general passes, which are slower on
+// every lattice tried: 100 x 75 x 50 403 -> 345 us for 20 steps, 17 x 90 x 33
+// 194 -> 166, 24^3 146 -> 136.)
+inline bool cubic_lean_taken(const sp_ctx *c)
 {
-    return c->lean && c->prec == SP_F32 && c->cubic && c->use_cubic && c->h.dipole == SP_DIPOLE_NONE &&
-           cubic_lean_fits(c->nc[0], c->nc[1], cubic_rows(c, pass));
+    return c->lean && c->prec == SP_F32 && c->cubic && c->use_cubic && c->h.dipole == SP_DIPOLE_NONE;
 }
+// Columns per thread of a lean pass: the user's choice, else two in the
+// predictor (which shares the rows both read and has two independent chains:
+// 1 to 7% faster on ten lattices from 24^3 to 128^3) and two in the corrector
+// where they make whole tiles (5% faster at 128^3, 13% at 64^3; on ragged
+// lattices 2 to 14% slower).
+inline int lean_rows(const sp_ctx *c, int pass)
+{
+    if (c->rows_set[0] || c->rows_set[1] || c->zc > 0 || c->zc_corr > 0) return c->rows[pass];
+    return pass == 0 || cubic_lean_fits(c->nc[0], c->nc[1], 2) ? 2 : 1;
+}
+inline int cubic_rows(const sp_ctx *c, int pass, bool lean) { return lean ? lean_rows(c, pass) : cubic_rows(c, pass); }
 
-// Units per CTA of the 27-point path: the user's choice, or the units spread
-// evenly over one wave of resident CTAs on the current device (units of the
-// pass's tile height, see cubic_rows).
-inline int cubic_per(sp_ctx *c, int pass = 0)
+inline int n_sms()
+{
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 1;
+    return nsm;
+}
+// Split of the 27-point path for a batch of n_rep replicas (of its lean passes:
+// lean): the user's choice, or all replicas' units spread over one wave of
+// resident CTAs (lean: runs of planes, see cubic_lean_runs; the corrector takes
+// the predictor's: 29 replicas of 30^3, 30 steps: 695 us, 702 with runs for its
+// own occupancy, 839 with the general passes).
+inline int cubic_per_batch(sp_ctx *c, int pass, int n_rep, bool lean)
 {
     if (pass == 1 && c->zc_corr > 0) return c->zc_corr;
     if (c->zc > 0) return c->zc;
-    int &a = pass == 0 ? c->zc_auto : c->zc_auto_corr;
+    if (lean)
+        return cubic_lean_runs(c->nc[0], c->nc[1], c->nc[2], 1, n_rep, n_sms(),
+                               cubic_lean_resident_ctas(0, 1, true, true));
+    long slots = (long)n_sms() * cubic_resident_ctas(c->prec, pass);
+    long units = cubic_units(c->nc[0], c->nc[1], c->nc[2]) * n_rep;
+    return (int)std::max(1L, (units + slots - 1) / slots);
+}
+
+// Units per CTA of the 27-point path (of its lean passes: lean): the user's
+// choice, or the units spread evenly over one wave of resident CTAs on the
+// current device (units of the pass's tile height, see cubic_rows).  (Cutting
+// every tile into runs, which suits a batch of replicas, gives a single lattice
+// too few CTAs: 100 x 75 x 50, 20 steps: 345 -> 456 us.)
+inline int cubic_per(sp_ctx *c, int pass, bool lean)
+{
+    if (pass == 1 && c->zc_corr > 0) return c->zc_corr;
+    if (c->zc > 0) return c->zc;
+    int &a = lean || !cubic_lean_taken(c) ? (pass == 0 ? c->zc_auto : c->zc_auto_corr) : c->zc_gen[pass != 0];
     if (a <= 0) {
-        int dev = 0, nsm = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 1;
-        const int rows = cubic_rows(c, pass);
-        long slots = (long)nsm * (cubic_lean_taken(c, pass) ? cubic_lean_resident_ctas(pass, rows)
-                                                             : cubic_resident_ctas(c->prec, pass, rows));
+        const int rows = cubic_rows(c, pass, lean);
+        const bool rag = !cubic_lean_fits(c->nc[0], c->nc[1], rows);
+        long slots = (long)n_sms() * (lean ? cubic_lean_resident_ctas(pass, rows, rag, false)
+                                           : cubic_resident_ctas(c->prec, pass, rows));
         long units = cubic_units(c->nc[0], c->nc[1], c->nc[2], rows);
         a = (int)std::max(1L, (units + slots - 1) / slots);
     }

@@ -544,10 +544,10 @@ cudaError_t launch_cubic(int pass, int solver, const CubicParams<T> &P, const re
                          rec_t<T> *nout, const rec_t<T> *Bdd, const LlgConst<T> &c, int per, cudaStream_t st, int rows,
                          bool lean)
 {
-    rows = cubic_rows_taken(sizeof(T) == 8 ? SP_F64 : SP_F32, rows, llg_reps(c) > 1, Bdd != nullptr);
     if constexpr (std::is_same<T, float>::value)
-        if (lean && solver == SP_HEUN && pass <= 1 && !Bdd && llg_reps(c) == 1 && cubic_lean_fits(P.nx, P.ny, rows))
+        if (lean && solver == SP_HEUN && pass <= 1 && !Bdd)
             return launch_cubic_lean(pass, P, src, np, q, nout, c, per, st, rows);
+    rows = cubic_rows_taken(sizeof(T) == 8 ? SP_F64 : SP_F32, rows, llg_reps(c) > 1, Bdd != nullptr);
     long total = cubic_units(P.nx, P.ny, P.nz, rows) * llg_reps(c);
     if (total == 0) return cudaSuccess;
     if (per < 1) per = 1;

@@ -1,7 +1,7 @@
 // cubic_lean.cu -- the stochastic Heun passes (App. B, Heun scheme with the
 // thermal field of the stochastic LLG equation) on the shell-symmetric
-// 27-point stencil, FP32, for one lattice without the dipole term whose xy
-// plane is cut into whole 32 x 8 column tiles (nx % 32 == 0, ny % 8 == 0).
+// 27-point stencil, FP32, for one lattice or a batch of replicas without the
+// dipole term.
 //
 // The plane streaming is that of cubic.cu: a CTA owns a 32 x 8 column tile
 // and a run of planes, planes pass through a ring of shared-memory tiles with
@@ -13,7 +13,9 @@
 //   * every tile record is read as one 16-byte vector and summed as two
 //     f32x2 halves (x, y | z, pad), so no load is split and every vector sum
 //     is two packed instructions;
-//   * whole tiles only: no per-spin ownership tests;
+//   * lattices cut into whole column tiles have kernels without per-spin
+//     ownership tests (ragged ones skip the stores of columns that do not
+//     exist);
 //   * the ring slot of every plane is a compile-time offset (the plane loop
 //     is unrolled by the ring size), staging addresses are fixed per segment
 //     and the halo slots that lie outside an open lattice are zeroed once
@@ -174,10 +176,10 @@ struct LeanRng {
     uint32_t yk;      // lo(M1 step_hi) ^ k0'           (round 1, first output word)
     uint32_t hk;      // hi(M0 x1) ^ k1'                (round 1, third output word)
     uint32_t l1;      // lo(M0 x1)                      (round 1, fourth output word)
-    uint32_t rk[16];  // round keys of rounds 2 .. 9
 };
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
-__device__ __forceinline__ uint4 lean_bits(const LeanRng &G, uint32_t i)
+// rk: the launch's round keys (those of rounds 2 .. 9 are read here)
+__device__ __forceinline__ uint4 lean_bits(const LeanRng &G, const uint32_t *rk, uint32_t i)
 {
     const uint32_t z1 = __umulhi(kPhiloxM0, i) ^ G.wk, w1 = kPhiloxM0 * i;
     uint4 c = make_uint4(__umulhi(kPhiloxM1, z1) ^ G.yk, kPhiloxM1 * z1, w1 ^ G.hk, G.l1);
@@ -185,23 +187,26 @@ __device__ __forceinline__ uint4 lean_bits(const LeanRng &G, uint32_t i)
     for (int r = 0; r < 8; ++r) {
         const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
         const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
-        c = make_uint4(hi1 ^ c.y ^ G.rk[2 * r], lo1, hi0 ^ c.w ^ G.rk[2 * r + 1], lo0);
+        c = make_uint4(hi1 ^ c.y ^ rk[4 + 2 * r], lo1, hi0 ^ c.w ^ rk[5 + 2 * r], lo0);
     }
     return c;
 }
-// the launch-uniform words of rounds 0 and 1 for the counter's step and
-// replica (x1 = round 0's first output word)
-LeanRng lean_rng(const LlgConst<float> &c)
+// the uniform words of rounds 0 and 1 for the counter's step and replica (x1 =
+// round 0's first output word): by the host for a launch of one lattice, by
+// each thread once per run of planes in a batch of replicas
+__host__ __device__ __forceinline__ uint32_t mulhi_u32(uint32_t a, uint32_t b)
 {
-    auto hi = [](uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); };
-    const uint32_t slo = (uint32_t)c.step, shi = (uint32_t)(c.step >> 32);
-    const uint32_t x1 = hi(kPhiloxM1, shi) ^ slo ^ c.rk[0], y1 = kPhiloxM1 * shi;
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+}
+__host__ __device__ __forceinline__ LeanRng lean_rng(const uint32_t *rk, uint64_t step, uint32_t replica)
+{
+    const uint32_t slo = (uint32_t)step, shi = (uint32_t)(step >> 32);
+    const uint32_t x1 = mulhi_u32(kPhiloxM1, shi) ^ slo ^ rk[0], y1 = kPhiloxM1 * shi;
     LeanRng G;
-    G.wk = (c.replica * 8u) ^ c.rk[1];
-    G.yk = y1 ^ c.rk[2];
-    G.hk = hi(kPhiloxM0, x1) ^ c.rk[3];
+    G.wk = (replica * 8u) ^ rk[1];
+    G.yk = y1 ^ rk[2];
+    G.hk = mulhi_u32(kPhiloxM0, x1) ^ rk[3];
     G.l1 = kPhiloxM0 * x1;
-    for (int k = 0; k < 16; ++k) G.rk[k] = c.rk[4 + k];
     return G;
 }
 
@@ -339,11 +344,12 @@ template <int R> struct LTile {
 // nout = n).  Plane p lives in ring slot (p - za + 1) % LNB; the LK planes
 // a group fetches form one cp.async group, waited for at the start of the
 // next group.
-template <int PASS, int DM, bool TH, int R>
+template <int PASS, int DM, bool TH, int R, bool RAG>
 __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const LeanConst &L, const LlgConst<float> &c,
                                              const float4 *__restrict__ src, float4 *__restrict__ np,
                                              float4 *__restrict__ q, float4 *__restrict__ nout, const LeanRng &G,
-                                             float4 *tiles, unsigned char *qt, int x0, int y0, int za, int zb)
+                                             float amp, float4 *tiles, unsigned char *qt, int x0, int y0, int za,
+                                             int zb)
 {
     constexpr int HN = LTile<R>::HN, NSL = LTile<R>::NSL;
     const int tid = threadIdx.x, tx = tid & (LX - 1), ty = tid / LX;
@@ -353,11 +359,13 @@ __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const 
     auto halo = [&](int e) {
         if (e >= HN) return -2;
         int gx = x0 - 1 + e % LHX, gy = y0 - 1 + e / LHX;
-        bool in = true;
+        // RAG: records past the first beyond the lattice belong to columns
+        // that do not exist
+        bool in = !RAG || (gx <= P.nx && gy <= P.ny);
         if (P.per0)
             gx = gx < 0 ? gx + P.nx : (gx >= P.nx ? gx - P.nx : gx);
         else
-            in = gx >= 0 && gx < P.nx;
+            in = in && gx >= 0 && gx < P.nx;
         if (P.per1)
             gy = gy < 0 ? gy + P.ny : (gy >= P.ny ? gy - P.ny : gy);
         else
@@ -377,6 +385,8 @@ __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const 
         for (int k = 0; k < NSL; ++k)
             if (g[k] == -1) st_zero(sd + b * kSlot + k * 16u * LT);
     const int col = (y0 + R * ty) * P.nx + x0 + tx;  // row 0 of the thread's strip
+    // columns of the thread that exist (rows 0 .. rows - 1 of its strip)
+    const int rows = !RAG ? R : (x0 + tx < P.nx ? min(R, max(0, P.ny - y0 - R * ty)) : 0);
     auto issue = [&](auto slot, int p) {
         constexpr unsigned S = decltype(slot)::value;
         if (p <= zb) {
@@ -401,6 +411,7 @@ __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const 
             if (PASS == 1 && p - 1 >= za && p - 1 < zb) {
 #pragma unroll
                 for (int j = 0; j < R; ++j) {
+                    if (RAG && j >= rows) continue;
                     const unsigned qs = qd + S * kQSlot + j * kQRec * LT;
                     const size_t qi = (size_t)(p - 1) * plane + col + j * P.nx;
                     if (SPGB_LEAN_PACKQ)
@@ -466,11 +477,12 @@ __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const 
             qx[j] = up[j].cw;
             if (PASS == 0) {
                 v3<float> Bth = mk(0.f, 0.f, 0.f);
-                if (TH) Bth = thermal(lean_bits(G, (uint32_t)ij), c.sig[0]);
+                if (TH) Bth = thermal(lean_bits(G, c.rk, (uint32_t)ij), amp);
                 const v3<float> A = lA(al, n, B + Bth);
                 const v3<float> f = cross(n, A);
                 const v3<float> p = unit(axpy(dt, f, n));
                 const v3<float> qv = TH ? axpy(hdt, f + cross(p, lA(al, p, Bth)), n) : axpy(hdt, f, n);
+                if (RAG && j >= rows) continue;
                 if (SPGB_LEAN_PACKQ) {
                     np[ij] = make_float4(p.x, p.y, p.z, qv.x);
                     q2[ij] = make_float2(qv.y, qv.z);
@@ -480,6 +492,7 @@ __device__ __forceinline__ void lean_segment(const CubicParams<float> &P, const 
                 }
             } else {
                 const v3<float> Ap = lA(al, n, B);
+                if (RAG && j >= rows) continue;
                 st(nout, ij, unit(axpy(hdt, cross(n, Ap), qi)));
             }
         }
@@ -518,9 +531,15 @@ template <int PASS, int R> struct LeanMinB {
                                         : (PASS == 0 ? SPGB_LEAN_MINB2 : SPGB_LEAN_MINB2_CORR);
 };
 
-// Work: the (32 x 8R column tile, plane) units in tile-major order, CTA b
-// takes units [b per, (b + 1) per) as runs of planes, one segment each.
-template <int PASS, int DM, bool TH, int R>
+// Work: the (32 x 8R column tile, plane) units in tile-major order (replica by
+// replica in a batch).  per > 0: CTA b takes units [b per, (b + 1) per) as
+// runs of planes, one segment each; per < 0: every tile's planes are cut into
+// -per runs of one segment (no run crosses a tile: a crossing reads two planes
+// more).
+// RAG: the extents are not those of whole tiles; the columns that do not exist
+// are computed (from zeros) and not stored.  REPL: a batch of replicas, each
+// with its noise amplitude and thermal stream.
+template <int PASS, int DM, bool TH, int R, bool RAG, bool REPL>
 __global__ void __launch_bounds__(LT, (LeanMinB<PASS, R>::value))
     k_lean(const __grid_constant__ CubicParams<float> P, const float4 *__restrict__ src, float4 *__restrict__ np,
            float4 *__restrict__ q, float4 *__restrict__ nout, const __grid_constant__ LlgConst<float> c,
@@ -530,24 +549,52 @@ __global__ void __launch_bounds__(LT, (LeanMinB<PASS, R>::value))
     __shared__ __align__(16) unsigned char qt[PASS == 1 ? LNB * LT * R * kQRec : 16];
     allow_dependents();
     wait_prerequisite();  // the previous pass wrote what this one reads
-    // units: (tile, plane) pairs, fewer than 2^31 (N < 2^31 spins, 256 R per
-    // tile and plane); one division per CTA, then the runs advance tile by tile
-    const int tiles_x = P.nx / LX;
-    const int total = tiles_x * (P.ny / (LY * R)) * P.nz;
-    int u = blockIdx.x * per;
-    const int u1 = min(u + per, total);
+    // units: (tile, plane) pairs, fewer than 2^31 (N < 2^31 spins, at least one
+    // per tile and plane); one division per CTA, then the runs advance tile by
+    // tile
+    const int tiles_x = RAG ? (P.nx + LX - 1) / LX : P.nx / LX;
+    const int tiles_y = RAG ? (P.ny + LY * R - 1) / (LY * R) : P.ny / (LY * R);
+    const int total = tiles_x * tiles_y * P.nz * (REPL ? c.n_rep : 1);
+    int u, u1;
+    if (per > 0) {
+        u = blockIdx.x * per;
+        u1 = (int)min((long long)u + per, (long long)total);
+    } else {
+        const int t = blockIdx.x / -per, r = blockIdx.x + t * per;
+        u = t * P.nz + (int)((long long)r * P.nz / -per);
+        u1 = t * P.nz + (int)((long long)(r + 1) * P.nz / -per);
+    }
     if (u >= u1) return;
-    const int tile = u / P.nz;
+    int tile = u / P.nz, rep = 0;
     int za = u - tile * P.nz;
+    if (REPL) {
+        rep = tile / (tiles_x * tiles_y);
+        tile -= rep * tiles_x * tiles_y;
+    }
     int ty = tile / tiles_x, tx = tile - ty * tiles_x;
+    const uint64_t step = REPL && TH ? llg_step_of(c) : 0;
     while (u < u1) {
         const int zb = min(P.nz, za + (u1 - u));
-        lean_segment<PASS, DM, TH, R>(P, L, c, src, np, q, nout, G, tiles, qt, tx * LX, ty * LY * R, za, zb);
+        if (REPL) {
+            const size_t o = (size_t)rep * P.nx * P.ny * P.nz;
+            const LeanRng Gr = TH ? lean_rng(c.rk, step, c.replica + (uint32_t)rep) : LeanRng{};
+            // (the packed q: 8 bytes per spin)
+            float4 *const qr = SPGB_LEAN_PACKQ ? reinterpret_cast<float4 *>(reinterpret_cast<float2 *>(q) + o) : q + o;
+            lean_segment<PASS, DM, TH, R, RAG>(P, L, c, src + o, PASS == 0 ? np + o : np, qr,
+                                               PASS == 1 ? nout + o : nout, Gr,
+                                               TH ? c.rsig[rep] * c.cA[0] : 0.f, tiles, qt, tx * LX, ty * LY * R, za, zb);
+        } else {
+            lean_segment<PASS, DM, TH, R, RAG>(P, L, c, src, np, q, nout, G, c.sig[0], tiles, qt, tx * LX, ty * LY * R, za,
+                                               zb);
+        }
         u += zb - za;
         za = 0;
         if (++tx == tiles_x) {
             tx = 0;
-            ++ty;
+            if (++ty == tiles_y && REPL) {
+                ty = 0;
+                ++rep;
+            }
         }
     }
 }
@@ -558,12 +605,15 @@ cudaError_t lean_launch(int grid, const CubicParams<float> &P, const float4 *src
 {
     const LeanConst L{make_float2(P.J1, P.J1), make_float2(P.J2, P.J2), make_float2(P.J3, P.J3),
                       make_float2(-1.f, -1.f)};
-    const LeanRng G = lean_rng(c);
-    if constexpr (PASS == 0)
-        if (c.thermal)
-            return launch_pdl(k_lean<PASS, DM, true, R>, dim3(grid), dim3(LT), 0, st, P, src, np, q, nout, c, L, G,
-                              per);
-    return launch_pdl(k_lean<PASS, DM, false, R>, dim3(grid), dim3(LT), 0, st, P, src, np, q, nout, c, L, G, per);
+    const LeanRng G = lean_rng(c.rk, c.step, c.replica);
+    const bool rag = !cubic_lean_fits(P.nx, P.ny, R), th = PASS == 0 && c.thermal;
+    constexpr bool TH = PASS == 0;  // the corrector has no thermal field
+    auto go = [&](auto kern) {
+        return launch_pdl(kern, dim3(grid), dim3(LT), 0, st, P, src, np, q, nout, c, L, G, per);
+    };
+    if (llg_reps(c) > 1) return th ? go(k_lean<PASS, DM, TH, R, true, true>) : go(k_lean<PASS, DM, false, R, true, true>);
+    if (rag) return th ? go(k_lean<PASS, DM, TH, R, true, false>) : go(k_lean<PASS, DM, false, R, true, false>);
+    return th ? go(k_lean<PASS, DM, TH, R, false, false>) : go(k_lean<PASS, DM, false, R, false, false>);
 }
 
 template <int PASS, int R>
@@ -573,6 +623,14 @@ cudaError_t lean_dm(int grid, const CubicParams<float> &P, const float4 *src, fl
     if (P.dmi_mode == 0) return lean_launch<PASS, 0, R>(grid, P, src, np, q, nout, c, per, st);
     if (P.dmi_mode == 1) return lean_launch<PASS, 1, R>(grid, P, src, np, q, nout, c, per, st);
     return lean_launch<PASS, 2, R>(grid, P, src, np, q, nout, c, per, st);
+}
+
+template <int PASS, int R> const void *lean_kernel(bool rag, bool repl)
+{
+    constexpr bool TH = PASS == 0;
+    return repl ? (const void *)k_lean<PASS, 1, TH, R, true, true>
+                : (rag ? (const void *)k_lean<PASS, 1, TH, R, true, false>
+                       : (const void *)k_lean<PASS, 1, TH, R, false, false>);
 }
 
 }  // namespace
@@ -586,10 +644,10 @@ cudaError_t launch_cubic_lean(int pass, const CubicParams<float> &P, const float
                               float4 *nout, const LlgConst<float> &c, int per, cudaStream_t st, int rows)
 {
     const int R = rows == 2 ? 2 : 1;
-    const long total = (long)(P.nx / LX) * (P.ny / (LY * R)) * P.nz;
+    const long total = cubic_units(P.nx, P.ny, P.nz, R) * llg_reps(c);
     if (total == 0) return cudaSuccess;
-    if (per < 1) per = 1;
-    const int grid = (int)((total + per - 1) / per);
+    if (per == 0) per = 1;
+    const int grid = (int)(per > 0 ? (total + per - 1) / per : total / P.nz * -per);
     // every field term and the noise amplitude in units of c = cA[0] (one
     // atom per cell): the kernels form c B directly
     const float s = c.cA[0];
@@ -613,16 +671,37 @@ cudaError_t launch_cubic_lean(int pass, const CubicParams<float> &P, const float
                      : lean_dm<1, 1>(grid, Ps, src, np, q, nout, cs, per, st);
 }
 
-int cubic_lean_resident_ctas(int pass, int rows)
+// Runs every tile's planes are cut into (see k_lean), as a negative split.  The
+// time of a pass is that of the SMs with the most work: m CTAs of p planes, each
+// with a prologue worth about 2.5 planes, an SM with one CTA a fifth slower per
+// plane than one with two (measured at 128^3: 0.88 and 0.72 us per 32 x 16
+// unit).  Best of all cuts with at most one wave of CTAs.
+// (Batches of replicas; against the units spread evenly over one wave, in runs
+// that cross tiles, 12 replicas of 30^3 take 439 us for 32 steps, not 498.)
+int cubic_lean_runs(int nx, int ny, int nz, int rows, int n_rep, int n_sm, int resident)
+{
+    if (nz <= 0) return -1;
+    const long tiles = cubic_units(nx, ny, 1, rows) * n_rep;
+    int best = 1;
+    double best_t = 1e300;
+    for (int runs = 1; runs <= nz; ++runs) {
+        const long m = (tiles * runs + n_sm - 1) / n_sm;
+        if (runs > 1 && m > resident) break;
+        const double t = (double)m * ((nz + runs - 1) / runs + 2.5) * (m == 1 ? 1.2 : 1.0);
+        if (t < best_t) {
+            best_t = t;
+            best = runs;
+        }
+    }
+    return -best;
+}
+
+int cubic_lean_resident_ctas(int pass, int rows, bool rag, bool replicas)
 {
     int n = 0;
-    cudaError_t e;
-    if (rows == 2)
-        e = pass == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lean<0, 1, true, 2>, LT, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lean<1, 1, false, 2>, LT, 0);
-    else
-        e = pass == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lean<0, 1, true, 1>, LT, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lean<1, 1, false, 1>, LT, 0);
+    const void *k = rows == 2 ? (pass == 0 ? lean_kernel<0, 2>(rag, replicas) : lean_kernel<1, 2>(rag, replicas))
+                              : (pass == 0 ? lean_kernel<0, 1>(rag, replicas) : lean_kernel<1, 1>(rag, replicas));
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, LT, 0);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }
 

@@ -58,6 +58,7 @@ template <typename T> int run_static(sp_ctx *c, void *n, const sp_llg_params *p,
     const Stencil<T> &S = *(const Stencil<T> *)(c->prec == SP_F64 ? (const void *)&c->Sd : (const void *)&c->Sf);
     const CubicParams<T> &CP = *(const CubicParams<T> *)(c->prec == SP_F64 ? (const void *)&c->Cd : (const void *)&c->Cf);
     bool cub = c->cubic && c->use_cubic && (p->solver == SP_HEUN || p->solver == SP_DEPONDT || p->solver == SP_SIB);
+    const bool lean = cub && p->solver == SP_HEUN && cubic_lean_taken(c);
     LlgConst<T> k{};
     k.dt = (T)p->dt;
     k.alpha = (T)p->alpha;
@@ -71,12 +72,12 @@ template <typename T> int run_static(sp_ctx *c, void *n, const sp_llg_params *p,
     k.thermal = (p->T > 0 && p->alpha > 0) ? 1 : 0;
     for (int s = 0; s < n_steps; ++s) {
         k.step = p->step0 + (uint64_t)s;
-        cudaError_t e = cub ? launch_cubic<T>(0, p->solver, CP, nn, np, q, nn, nullptr, k, cubic_per(c), st,
-                                              cubic_rows(c, 0), cubic_lean_taken(c, 0))
+        cudaError_t e = cub ? launch_cubic<T>(0, p->solver, CP, nn, np, q, nn, nullptr, k, cubic_per(c, 0, lean), st,
+                                              cubic_rows(c, 0, lean), lean)
                             : launch_llg_pred<T>(p->solver, S, nn, nullptr, np, q, k, st);
         if (e == cudaSuccess)
-            e = cub ? launch_cubic<T>(1, p->solver, CP, np, nullptr, q, nn, nullptr, k, cubic_per(c, 1), st,
-                                      cubic_rows(c, 1), cubic_lean_taken(c, 1))
+            e = cub ? launch_cubic<T>(1, p->solver, CP, np, nullptr, q, nn, nullptr, k, cubic_per(c, 1, lean), st,
+                                      cubic_rows(c, 1, lean), lean)
                     : launch_llg_corr<T>(p->solver, S, nn, np, q, nullptr, k, st);
         if (e != cudaSuccess) {
             c->err = std::string("LLG launch: ") + cudaGetErrorString(e);
