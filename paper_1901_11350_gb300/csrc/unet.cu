@@ -903,6 +903,11 @@ __global__ void __launch_bounds__(128) k_wgrad(ConvSrc S, const bf16 *__restrict
 // runs).  The FP32 accumulator (128 lanes x BN columns of tensor memory) is
 // this split's partial sum part[z][co][t][ci]; k_sum_parts adds the splits
 // in a fixed order.  Waits are bounded as in k_conv_tc.
+// Where 9 Cin is not a multiple of 128 the last row tile has rows to spare:
+// row 9 Cin of A is all ones, and its accumulator is the split's part of the
+// bias gradient, bias_part[z][co] (one more read of dz otherwise, 67 MB at
+// 64 x 128^2 x 32 channels: the column sums of a training step took 210 us, 95
+// are left).
 constexpr int kWgPix = 32;  // pixels per stage
 
 template <int BN>
@@ -923,7 +928,8 @@ __device__ __forceinline__ uint64_t desc_mn64(unsigned addr, unsigned lbo, unsig
 
 template <int BN>
 __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__restrict__ dz, int H, int W, int Cout,
-                                                       int P, int pix_per_split, float *__restrict__ part)
+                                                       int P, int pix_per_split, float *__restrict__ part,
+                                                       float *__restrict__ bias_part)
 {
     constexpr int NA = BN / 32;                 // channel runs (atoms) of the B tile
     constexpr int A_BYTES = 4 * 4 * 512;        // 4 runs x 4 pixel groups
@@ -1008,9 +1014,13 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__
     for (int s = 0; s < kTcStages; ++s)
         for (int i = tid; i < 4 * 128; i += kThreads) {
             const int run = i >> 7;
-            if (m0 + 32 * run >= R)
-                *reinterpret_cast<uint4 *>(smem_raw + (base - raw) + s * STAGE + run * 2048 + (i & 127) * 16) =
-                    make_uint4(0u, 0u, 0u, 0u);
+            if (m0 + 32 * run >= R) {
+                // byte offset of 16-byte chunk c of pixel px in the run
+                const int px = (i & 127) >> 2, c = i & 3;
+                const unsigned one = m0 + 32 * run == R && c == 0 ? 0x3F80u : 0u;  // channel 0: BF16 1.0
+                *reinterpret_cast<uint4 *>(smem_raw + (base - raw) + s * STAGE + run * 2048 + (px >> 3) * 512 +
+                                           swz64(px & 7, c)) = make_uint4(one, 0u, 0u, 0u);
+            }
         }
     tc_fence_before();
     __syncthreads();
@@ -1061,10 +1071,16 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__
     for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 16) {
         float v[16];
         tc_ld16(tmem + ((unsigned)(q * 32) << 16) + (unsigned)c0, v);
-        if (failed || r >= R) continue;
+        if (failed || r > R) continue;
         if (nk == 0) {
 #pragma unroll
             for (int e = 0; e < 16; ++e) v[e] = 0.f;
+        }
+        if (r == R) {
+            if (bias_part)
+#pragma unroll
+                for (int e = 0; e < 16; ++e) bias_part[(size_t)blockIdx.z * Cout + n0 + c0 + e] = v[e];
+            continue;
         }
 #pragma unroll
         for (int e = 0; e < 16; ++e) pz[((size_t)(n0 + c0 + e) * 9 + t) * Cin + ci] = v[e];
@@ -1076,20 +1092,40 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__
     if (failed && tid == 0) atomicExch(&g_tc_error, 1);
 }
 
-// out[i] = sum_{z < nz} part[z * n + i], in order of z.
-__global__ void k_sum_parts(const float *__restrict__ part, int nz, long long n, float *__restrict__ out)
+// out[i] = sum_{z < nz} part[z * n + i].  A block takes 256 / G values, G
+// threads each: thread g sums z = g, g + G, ... in four running sums (four
+// loads in flight), added as (s0 + s1) + (s2 + s3), and the G sums are added
+// in order: fixed for a given (nz, n).  What bounds it is the chain of loads
+// of a thread: with one thread per value (G = 1) 253 partials are 64
+// trips to memory one after another (28 launches of a training step: 204 us; the 24 that
+// take eight threads now 111).
+template <int G>
+__global__ void __launch_bounds__(256) k_sum_parts(const float *__restrict__ part, int nz, long long n,
+                                                   float *__restrict__ out)
 {
-    // four running sums over z = 4k + j (four loads in flight), added as
-    // (s0 + s1) + (s2 + s3): a fixed order
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    constexpr int V = 256 / G;
+    __shared__ float sh[G > 1 ? 256 : 1];
+    const int g = threadIdx.x / V, l = threadIdx.x % V;
+    for (long long i0 = blockIdx.x * (long long)V; i0 < n; i0 += (long long)gridDim.x * V) {
+        const long long i = i0 + l;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
-        int z = 0;
-        for (; z + 3 < nz; z += 4) {
+        if (i < n) {
+            int z = g;
+            for (; z + 3 * G < nz; z += 4 * G) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) s[j] += __ldg(part + (size_t)(z + j) * n + i);
+                for (int j = 0; j < 4; ++j) s[j] += __ldg(part + (size_t)(z + j * G) * n + i);
+            }
+            for (int j = 0; z < nz; z += G, ++j) s[j] += __ldg(part + (size_t)z * n + i);
         }
-        for (int j = 0; z < nz; ++z, ++j) s[j] += __ldg(part + (size_t)z * n + i);
-        out[i] = (s[0] + s[1]) + (s[2] + s[3]);
+        float t = (s[0] + s[1]) + (s[2] + s[3]);
+        if (G > 1) {
+            sh[threadIdx.x] = t;
+            __syncthreads();
+            if (g == 0)
+                for (int k = 1; k < G; ++k) t += sh[k * V + l];
+            __syncthreads();
+        }
+        if (g == 0 && i < n) out[i] = t;
     }
 }
 
@@ -1607,9 +1643,20 @@ long long wgrad_ws_bytes(long long P, int Cin, int Cout)
     return b;
 }
 
+// Eight threads per value from 32 partials on: below, the loads of one thread
+// are few enough.
+cudaError_t sum_parts(const float *part, int nz, long long n, float *out, cudaStream_t st)
+{
+    if (nz >= 32)
+        k_sum_parts<8><<<(unsigned)std::min((n + 31) / 32, 4096LL), 256, 0, st>>>(part, nz, n, out);
+    else
+        k_sum_parts<1><<<grid_for(n), 256, 0, st>>>(part, nz, n, out);
+    return cudaGetLastError();
+}
+
 template <int BN>
 cudaError_t wgrad_tc_launch(dim3 grid, const ConvSrc &S, const bf16 *dz, int H, int Wd, int Cout, int P, int pps,
-                            float *part, cudaStream_t st)
+                            float *part, float *bias_part, cudaStream_t st)
 {
     static bool attr = false;  // per process; the attribute is per function
     constexpr size_t sm = wgrad_tc_smem<BN>();
@@ -1618,7 +1665,7 @@ cudaError_t wgrad_tc_launch(dim3 grid, const ConvSrc &S, const bf16 *dz, int H, 
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    k_wgrad_tc<BN><<<grid, kThreads, sm, st>>>(S, dz, H, Wd, Cout, P, pps, part);
+    k_wgrad_tc<BN><<<grid, kThreads, sm, st>>>(S, dz, H, Wd, Cout, P, pps, part, bias_part);
     return cudaGetLastError();
 }
 
@@ -1628,14 +1675,18 @@ cudaError_t wgrad_launch(const ConvSrc &S, const bf16 *dz, int B, int H, int Wd,
     long long P = (long long)B * H * Wd;
     int Cin = S.C0 + S.C1;
     WgradPlan w = wgrad_plan(P, Cin, Cout, g_use_tc != 0);
+    // the tensor cores sum the bias gradient too where a row tile has a row to
+    // spare (and the splits' parts fit the workspace)
+    const bool fold = db && w.tc_bn && (9 * Cin) % 128 != 0 && w.splits <= w.bias_blocks;
+    float *bp = ws + w.part_floats, *fp = fold ? bp : nullptr;
     if (w.tc_bn) {
         dim3 grid((unsigned)((9 * Cin + 127) / 128), (unsigned)(Cout / w.tc_bn), (unsigned)w.splits);
         cudaError_t e;
         switch (w.tc_bn) {
-        case 256: e = wgrad_tc_launch<256>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, st); break;
-        case 128: e = wgrad_tc_launch<128>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, st); break;
-        case 64: e = wgrad_tc_launch<64>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, st); break;
-        default: e = wgrad_tc_launch<32>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, st); break;
+        case 256: e = wgrad_tc_launch<256>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, fp, st); break;
+        case 128: e = wgrad_tc_launch<128>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, fp, st); break;
+        case 64: e = wgrad_tc_launch<64>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, fp, st); break;
+        default: e = wgrad_tc_launch<32>(grid, S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws, fp, st); break;
         }
         if (e != cudaSuccess) return e;
     } else {
@@ -1646,12 +1697,12 @@ cudaError_t wgrad_launch(const ConvSrc &S, const bf16 *dz, int B, int H, int Wd,
             k_wgrad<32><<<grid, 128, 0, st>>>(S, dz, H, Wd, Cout, (int)P, w.pix_per_split, ws);
     }
     long long n = (long long)Cout * 9 * Cin;
-    k_sum_parts<<<grid_for(n), 256, 0, st>>>(ws, w.splits, n, dW);
-    if (db) {
-        float *bp = ws + w.part_floats;
+    cudaError_t e = sum_parts(ws, w.splits, n, dW, st);
+    if (e != cudaSuccess || !db) return e;
+    if (!fold)
         k_colsum<<<dim3(w.bias_blocks, (Cout + 255) / 256), 256, 0, st>>>(dz, (int)P, Cout, w.bias_pix, bp);
-        k_sum_parts<<<grid_for(Cout), 256, 0, st>>>(bp, w.bias_blocks, Cout, db);
-    }
+    e = sum_parts(bp, fold ? w.splits : w.bias_blocks, Cout, db, st);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
