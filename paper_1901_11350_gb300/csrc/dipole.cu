@@ -204,7 +204,7 @@ struct DipolePlan {
          *tw1[2] = {nullptr, nullptr};
     bool ready[2] = {false, false};
     // FP32 warp-FFT path on a 1024 x 1024 grid
-    bool fast = false, force_generic = false;
+    bool fast = false, planar = false, force_generic = false;
     void *Kt = nullptr, *ST = nullptr;
 };
 
@@ -272,7 +272,10 @@ template <typename T> cudaError_t prepare(DipolePlan *p, cudaStream_t st)
             grid[4 * M + o] = 3 * u[1] * u[2] * i3;
             grid[5 * M + o] = (3 * u[2] * u[2] - 1) * i3;
         }
+    // a film in the xy plane: xz and yz vanish, and so do their transforms
+    const bool planar = p->g.A[0][2] == 0.0 && p->g.A[1][2] == 0.0;
     for (int c = 0; c < 6; ++c) {
+        if (planar && (c == 2 || c == 4)) continue;
         std::complex<double> *a = grid.data() + c * M;
         for (int g1 = 0; g1 < d.P1; ++g1) host_fft(a + (long)g1 * d.P0, d.P0, 1);
         if (d.P1 > 1)
@@ -285,11 +288,14 @@ template <typename T> cudaError_t prepare(DipolePlan *p, cudaStream_t st)
             for (int c = 0; c < 6; ++c) K[((size_t)ky * d.ncols + kx) * 6 + c] = (T)(grid[c * M + (long)ky * d.P0 + kx].real() * scale);
     if (sizeof(T) == 4 && d.P0 == 1024 && d.P1 == 1024) {
         // per-column structure of arrays for the warp-FFT path: Kt[kx][6][ky]
-        std::vector<float> Kt((size_t)513 * 1024 * 6);
+        // (planar: without the components that vanish, see dipole_fast_run)
+        std::vector<int> comp = planar ? std::vector<int>{0, 1, 3, 5} : std::vector<int>{0, 1, 2, 3, 4, 5};
+        std::vector<float> Kt((size_t)513 * 1024 * comp.size());
         for (int kx = 0; kx < 513; ++kx)
-            for (int c = 0; c < 6; ++c)
+            for (size_t c = 0; c < comp.size(); ++c)
                 for (int ky = 0; ky < 1024; ++ky)
-                    Kt[((size_t)kx * 6 + c) * 1024 + ky] = (float)(grid[c * M + (long)ky * d.P0 + kx].real() * scale);
+                    Kt[((size_t)kx * comp.size() + c) * 1024 + ky] =
+                        (float)(grid[comp[c] * M + (long)ky * d.P0 + kx].real() * scale);
         cudaError_t e;
         if ((e = cudaMalloc(&p->Kt, sizeof(float) * Kt.size())) != cudaSuccess) return e;
         if ((e = cudaMalloc(&p->ST, sizeof(float2) * 3 * 513 * (size_t)d.n1)) != cudaSuccess) return e;
@@ -297,6 +303,7 @@ template <typename T> cudaError_t prepare(DipolePlan *p, cudaStream_t st)
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
         if ((e = dipole_fast_setup()) != cudaSuccess) return e;
         p->fast = true;
+        p->planar = planar;
     }
     std::vector<C> t0(std::max(1, d.P0 / 2)), t1(std::max(1, d.P1 / 2));
     for (int k = 0; k < d.P0 / 2; ++k) t0[k] = C{(T)std::cos(2 * M_PI * k / d.P0), (T)-std::sin(2 * M_PI * k / d.P0)};
@@ -327,7 +334,8 @@ template <typename T> cudaError_t run(DipolePlan *p, const void *n, void *out, c
     using C = cx_t<T>;
     const Dims &d = p->d;
     if (sizeof(T) == 4 && p->fast && !p->force_generic)
-        return dipole_fast_run(d.n0, d.n1, (const float4 *)n, (float2 *)p->ST, (const float *)p->Kt, (float4 *)out, st);
+        return dipole_fast_run(d.n0, d.n1, (const float4 *)n, (float2 *)p->ST, (const float *)p->Kt, p->planar,
+                               (float4 *)out, st);
     size_t row_smem = 2 * sizeof(C) * d.P0, col_smem = 3 * sizeof(C) * (size_t)d.cw * d.P1;
     C *S = (C *)p->S[ix];
     k_dip_rows<T><<<d.n1, 256, row_smem, st>>>(d, (const rec_t<T> *)n, S, (const C *)p->tw0[ix]);

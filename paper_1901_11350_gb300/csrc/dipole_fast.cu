@@ -10,7 +10,16 @@
 //   pass reads and writes coalesced runs, and the row passes move runs of
 //   two rows;
 // * the column pass multiplies by Khat in the strided register layout the
-//   inverse transform takes as input, so no reordering is needed.
+//   inverse transform takes as input, so no reordering is needed;
+// * a film in the xy plane (every Bravais vector in the plane) has
+//   Khat_xz = Khat_yz = 0: the column pass of such a plan reads four of the six
+//   components, and its z warp multiplies its own registers.
+// What bounds the passes is the latency of one wave of few warps (two row
+// blocks per SM, 3.4 columns per SM), so whatever does not depend on the pass
+// before -- the column's Khat and the table of the four-step twiddles, 8 KB in
+// shared memory -- is fetched before the wait for it.  (512 x 512, 40
+// evaluations and steps: 1287 -> 1271 us; and the first call transforms four
+// components on the host instead of six.)
 #include <cmath>
 
 #include "dipole.h"
@@ -96,12 +105,14 @@ __device__ float2 g_tw1024[32 * 32];
 // Four-step 1024-point FFT by one warp: on entry a[n2] = x[32 n2 + lane], on
 // exit a[k1] = X[lane + 32 k1].  tr: this warp's 32 x 33 transpose tile.
 // ZIN: x[512..1023] = 0 (a[16..31] are not read).
-template <bool INV, bool ZIN = false> __device__ __forceinline__ void fft1024(float2 (&a)[32], float2 *tr, int lane)
+// tw: g_tw1024, or its copy in shared memory.
+template <bool INV, bool ZIN = false>
+__device__ __forceinline__ void fft1024(float2 (&a)[32], float2 *tr, int lane, const float2 *tw)
 {
     fft32<INV, ZIN>(a);
 #pragma unroll
     for (int k2 = 1; k2 < 32; ++k2) {
-        const float2 w = __ldg(&g_tw1024[k2 * 32 + lane]);
+        const float2 w = tw[k2 * 32 + lane];
         a[k2] = cm(a[k2], INV ? cj(w) : w);
     }
 #pragma unroll
@@ -111,6 +122,26 @@ template <bool INV, bool ZIN = false> __device__ __forceinline__ void fft1024(fl
     for (int n1 = 0; n1 < 32; ++n1) a[n1] = tr[lane * 33 + n1];
     __syncwarp();
     fft32<INV>(a);
+}
+
+__device__ __forceinline__ void cp16(void *smem, const void *gmem)
+{
+    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
+}
+__device__ __forceinline__ void cp8(void *smem, const void *gmem)
+{
+    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+}
+
+constexpr int kTw = 32 * 32;  // four-step twiddles
+// The twiddle table into shared memory (asynchronously; the block's first
+// barrier after its cp.async wait publishes it).
+__device__ __forceinline__ void stage_twiddles(float2 *tw)
+{
+    for (int t = threadIdx.x; t < kTw / 2; t += blockDim.x) cp16(tw + 2 * t, g_tw1024 + 2 * t);
+    asm volatile("cp.async.commit_group;\n" ::);
 }
 
 // ------------------------------------------------------------ row pass
@@ -126,7 +157,11 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
     int w = wid >> 1, part = wid & 1;  // row in block; 0: z, 1: x + i y
     int y0 = blockIdx.x * kRows, y = y0 + w;
     bool row = y < n1;
+    float2 *tw = sm + 3 * 513 * kRows + 2 * kRows * kTr;
     allow_dependents();
+    stage_twiddles(tw);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
     wait_prerequisite();  // the spins may come from the pass just before
     float2 a[32];
 #pragma unroll
@@ -136,7 +171,7 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
         a[n2] = part ? make_float2(v.x, v.y) : make_float2(v.z, 0.f);
         a[n2 + 16] = make_float2(0.f, 0.f);
     }
-    fft1024<false, true>(a, tr, lane);
+    fft1024<false, true>(a, tr, lane, tw);
     if (part == 0) {
 #pragma unroll
         for (int k1 = 0; k1 <= 16; ++k1) {
@@ -172,32 +207,34 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
 // the forward transform over y runs (zero rows y >= n1); product with Khat
 // in the strided layout of the inverse transform's input; rows y < n1
 // written back in place.
-__device__ __forceinline__ void cp16(void *smem, const void *gmem)
-{
-    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void cp8(void *smem, const void *gmem)
-{
-    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
-}
+// Barrier of the x and y warps.
+__device__ __forceinline__ void xy_barrier() { asm volatile("bar.sync 1, 64;\n" ::: "memory"); }
 
+template <bool PLANAR>
 __global__ void __launch_bounds__(96) k_cols(int n1, float2 *__restrict__ ST, const float *__restrict__ Kt)
 {
     // The transpose tiles are live only inside the transforms and the spectra
     // only between them, so they share memory (barriers between the phases):
-    // 49 KB per block, four blocks per SM, all 513 columns in one wave.
+    // 49 KB per block, four blocks per SM, all 513 columns in one wave (four
+    // components of Khat and the twiddles, or all six and the twiddles from L1).
+    constexpr int NK = PLANAR ? 4 : 6;
     extern __shared__ float2 sm[];
     float2 *spec = sm;                                  // [3][1024], between the transforms
     float2 *tr = sm + (threadIdx.x / 32) * kTr;         // [3][kTr], inside the transforms
-    float *ks = reinterpret_cast<float *>(sm + 3 * kTr);  // [6][1024]
+    float *ks = reinterpret_cast<float *>(sm + 3 * kTr);  // [NK][1024]
+    float2 *tws = reinterpret_cast<float2 *>(ks + NK * 1024);
+    const float2 *tw = PLANAR ? tws : g_tw1024;
     int c = threadIdx.x / 32, lane = threadIdx.x % 32;
     int kx = blockIdx.x;
-    const float *K = Kt + (long)kx * 6 * 1024;
+    const float *K = Kt + (long)kx * NK * 1024;
     allow_dependents();
-    for (int t = threadIdx.x; t < 6 * 1024 / 4; t += blockDim.x) cp16(ks + 4 * t, K + 4 * t);
+    if (PLANAR) stage_twiddles(tws);
+    for (int t = threadIdx.x; t < NK * 1024 / 4; t += blockDim.x) cp16(ks + 4 * t, K + 4 * t);
     asm volatile("cp.async.commit_group;\n" ::);
+    if (PLANAR) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();
+    }
     wait_prerequisite();  // the row spectra
     float2 *col = ST + ((long)c * 513 + kx) * n1;
     float2 a[32];
@@ -207,25 +244,49 @@ __global__ void __launch_bounds__(96) k_cols(int n1, float2 *__restrict__ ST, co
         a[n2] = y < n1 ? col[y] : make_float2(0.f, 0.f);
         a[n2 + 16] = make_float2(0.f, 0.f);
     }
-    fft1024<false, true>(a, tr, lane);
-    __syncthreads();  // every warp is done with its transpose tile
+    fft1024<false, true>(a, tr, lane, tw);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();  // Khat has landed; every warp is done with its transpose tile
+    if (PLANAR) {
+        // components xx xy yy zz; the spectrum of a warp is in the layout its
+        // inverse transform takes
+        if (c == 2) {
 #pragma unroll
-    for (int k1 = 0; k1 < 32; ++k1) spec[c * 1024 + lane + 32 * k1] = a[k1];
-    asm volatile("cp.async.wait_group 0;\n" ::);
-    __syncthreads();
-    // row c of the symmetric tensor (xx xy xz yy yz zz)
-    const int i0 = c == 0 ? 0 : (c == 1 ? 1 : 2);
-    const int i1 = c == 0 ? 1 : (c == 1 ? 3 : 4);
-    const int i2 = c == 0 ? 2 : (c == 1 ? 4 : 5);
+            for (int n2 = 0; n2 < 32; ++n2) {
+                const float r = ks[3 * 1024 + 32 * n2 + lane];
+                a[n2] = make_float2(r * a[n2].x, r * a[n2].y);
+            }
+        } else {
 #pragma unroll
-    for (int n2 = 0; n2 < 32; ++n2) {
-        int ky = 32 * n2 + lane;
-        float r0 = ks[i0 * 1024 + ky], r1 = ks[i1 * 1024 + ky], r2 = ks[i2 * 1024 + ky];
-        float2 X = spec[ky], Y = spec[1024 + ky], Z = spec[2048 + ky];
-        a[n2] = make_float2(r0 * X.x + r1 * Y.x + r2 * Z.x, r0 * X.y + r1 * Y.y + r2 * Z.y);
+            for (int k1 = 0; k1 < 32; ++k1) spec[c * 1024 + lane + 32 * k1] = a[k1];
+            xy_barrier();
+#pragma unroll
+            for (int n2 = 0; n2 < 32; ++n2) {
+                const int ky = 32 * n2 + lane;
+                const float r0 = ks[c * 1024 + ky], r1 = ks[(c + 1) * 1024 + ky];
+                const float2 o = spec[(1 - c) * 1024 + ky], X = c == 0 ? a[n2] : o, Y = c == 0 ? o : a[n2];
+                a[n2] = make_float2(r0 * X.x + r1 * Y.x, r0 * X.y + r1 * Y.y);
+            }
+            xy_barrier();  // both have read the spectra before the tiles reuse them
+        }
+    } else {
+#pragma unroll
+        for (int k1 = 0; k1 < 32; ++k1) spec[c * 1024 + lane + 32 * k1] = a[k1];
+        __syncthreads();
+        // row c of the symmetric tensor (xx xy xz yy yz zz)
+        const int i0 = c == 0 ? 0 : (c == 1 ? 1 : 2);
+        const int i1 = c == 0 ? 1 : (c == 1 ? 3 : 4);
+        const int i2 = c == 0 ? 2 : (c == 1 ? 4 : 5);
+#pragma unroll
+        for (int n2 = 0; n2 < 32; ++n2) {
+            int ky = 32 * n2 + lane;
+            float r0 = ks[i0 * 1024 + ky], r1 = ks[i1 * 1024 + ky], r2 = ks[i2 * 1024 + ky];
+            float2 X = spec[ky], Y = spec[1024 + ky], Z = spec[2048 + ky];
+            a[n2] = make_float2(r0 * X.x + r1 * Y.x + r2 * Z.x, r0 * X.y + r1 * Y.y + r2 * Z.y);
+        }
+        __syncthreads();  // every warp has read the spectra before the tiles reuse them
     }
-    __syncthreads();  // every warp has read the spectra before the tiles reuse them
-    fft1024<true>(a, tr, lane);
+    fft1024<true>(a, tr, lane, tw);
 #pragma unroll
     for (int k1 = 0; k1 < 16; ++k1) {
         int y = lane + 32 * k1;
@@ -245,7 +306,9 @@ __global__ void __launch_bounds__(64 * kRows) k_irows(int n0, int n1, const floa
     int wid = threadIdx.x / 32, lane = threadIdx.x % 32;
     int w = wid >> 1, part = wid & 1;
     int y0 = blockIdx.x * kRows, y = y0 + w;
+    float2 *tw = reinterpret_cast<float2 *>(zs + kRows * 512);
     allow_dependents();
+    stage_twiddles(tw);
     wait_prerequisite();  // the column pass's spectra
     for (int t = threadIdx.x; t < 3 * 513 * kRows; t += blockDim.x) {
         int r = t % kRows, ck = t / kRows;
@@ -275,7 +338,7 @@ __global__ void __launch_bounds__(64 * kRows) k_irows(int n0, int n1, const floa
             a[n2] = make_float2(X.x - Y.y, X.y + Y.x);  // X + i Y
         }
     }
-    fft1024<true>(a, tr, lane);
+    fft1024<true>(a, tr, lane, tw);
     if (part == 0) {
 #pragma unroll
         for (int k1 = 0; k1 < 16; ++k1) zs[w * 512 + lane + 32 * k1] = a[k1].x;
@@ -290,8 +353,11 @@ __global__ void __launch_bounds__(64 * kRows) k_irows(int n0, int n1, const floa
     }
 }
 
-constexpr size_t kRowSmem = sizeof(float2) * (3 * 513 * kRows + 2 * kRows * kTr) + sizeof(float) * kRows * 512;
+constexpr size_t kRowSmem = sizeof(float2) * (3 * 513 * kRows + 2 * kRows * kTr + kTw);
+constexpr size_t kIrowSmem = kRowSmem + sizeof(float) * kRows * 512;
 constexpr size_t kColSmem = sizeof(float2) * (3 * kTr) + sizeof(float) * 6 * 1024;
+constexpr size_t kColSmemPlanar = sizeof(float2) * (3 * kTr + kTw) + sizeof(float) * 4 * 1024;
+static_assert((3 * 513 * kRows + 2 * kRows * kTr) % 2 == 0 && (kRows * 512) % 4 == 0, "16-byte copies of the twiddles");
 static_assert(3 * kTr >= 3 * 1024, "the transpose tiles must cover the spectra they alias");
 
 }  // namespace
@@ -311,17 +377,23 @@ cudaError_t dipole_fast_setup()
         table = true;
     }
     cudaError_t e = cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_irows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_irows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIrowSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColSmemPlanar);
     return e;
 }
 
-cudaError_t dipole_fast_run(int n0, int n1, const float4 *n, float2 *ST, const float *Kt, float4 *out, cudaStream_t st)
+cudaError_t dipole_fast_run(int n0, int n1, const float4 *n, float2 *ST, const float *Kt, bool planar, float4 *out,
+                            cudaStream_t st)
 {
     int rb = (n1 + kRows - 1) / kRows;
     cudaError_t e = launch_pdl(k_rows, dim3(rb), dim3(64 * kRows), kRowSmem, st, n0, n1, n, ST);
-    if (e == cudaSuccess) e = launch_pdl(k_cols, dim3(513), dim3(96), kColSmem, st, n1, ST, Kt);
-    if (e == cudaSuccess) e = launch_pdl(k_irows, dim3(rb), dim3(64 * kRows), kRowSmem, st, n0, n1, (const float2 *)ST, out);
+    if (e == cudaSuccess)
+        e = planar ? launch_pdl(k_cols<true>, dim3(513), dim3(96), kColSmemPlanar, st, n1, ST, Kt)
+                   : launch_pdl(k_cols<false>, dim3(513), dim3(96), kColSmem, st, n1, ST, Kt);
+    if (e == cudaSuccess) e = launch_pdl(k_irows, dim3(rb), dim3(64 * kRows), kIrowSmem, st, n0, n1, (const float2 *)ST, out);
     return e;
 }
 

@@ -9,7 +9,9 @@ namespace spgb {
 cudaError_t dipole_fast_setup();
 // Field of the spins n (n0 x n1, 257..512 per side) into out; ST: 3 x 513 x n1
 // complex scratch; Kt: transformed kernel [513][6][1024] (structure of arrays
-// per column), scaled.
-cudaError_t dipole_fast_run(int n0, int n1, const float4 *n, float2 *ST, const float *Kt, float4 *out, cudaStream_t st);
+// per column; xx xy xz yy yz zz), scaled; planar (xz = yz = 0): [513][4][1024]
+// (xx xy yy zz).
+cudaError_t dipole_fast_run(int n0, int n1, const float4 *n, float2 *ST, const float *Kt, bool planar, float4 *out,
+                            cudaStream_t st);
 
 }  // namespace spgb

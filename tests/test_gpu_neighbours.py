@@ -118,3 +118,19 @@ def test_sampled_observables_of_many_blocks(L, R):
         m = np.linalg.norm(n0[r].sum(axis=0)) / c.N
         want = np.array([m, m * m, m ** 4, E, E * E, 1, 0, 0])
         assert np.all(np.abs(st[r] - want) <= 1e-6 * np.abs(want) * np.array([1, 2, 4, 1, 2, 0, 0, 0]))
+
+
+@pytest.mark.parametrize("tilt", [0.0, 0.4])
+@pytest.mark.parametrize("n0,n1", [(257, 512), (400, 301)])
+def test_dipole_columns_of_films_in_and_out_of_the_plane(tilt, n0, n1):
+    # a film in the xy plane has no xz and yz components, a tilted one all six
+    # (the bound of the direct sum in test_gpu_parity.py)
+    g = I.hexagonal(n0, n1, mu_s=3.0)
+    g = dict(g, bravais=[g["bravais"][0], [g["bravais"][1][0], g["bravais"][1][1], tilt], g["bravais"][2]])
+    n = I.random_spins(n0 * n1, 13)
+    c = B.Context(g, dict(J=[1.0], dipole="fft"), "f32")
+    Bf = _np(c.effective_field(c.spins(n)))
+    o = oracle.System(g, dict(J=[1.0], dipole="direct"))
+    idx = np.concatenate([np.random.default_rng(1).choice(o.N, 60, replace=False), [0, n0 - 1, o.N - 1]])
+    ref = o.field(n, dipole="none")[idx] + o.dipole_field_direct_at(n, idx)
+    assert np.abs(Bf[idx] - ref).max() <= 1e-5 * np.abs(ref).max()
