@@ -1092,6 +1092,162 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__
     if (failed && tid == 0) atomicExch(&g_tc_error, 1);
 }
 
+// ------------------------------------------------------------------ wgrad, tcgen05, halo tiles
+// The weight gradient with the input of a band of R image rows staged once per
+// 32 input channels (k_wgrad_tc copies every tap's shifted rows: nine times the
+// input).  A CTA takes 32 channels ci, BN output channels and the bands of one
+// split.  Both operands are MN-major without swizzle: planes of 8 channels, 16
+// bytes per pixel, so that along K (pixels) the two 8-pixel groups of an MMA
+// are neighbours and a shift by one pixel is a 16-byte aligned start address.
+// The planes of a row of the input tile (R + 2 rows of W + 2 pixels) follow one
+// another and the next row's follow them: 16 planes are four rows, and one MMA
+// over the pixels of output row y,
+//     D_dx[32 r + ci][co] += sum_x in[y + r - 1][x + dx - 1][ci] dz[y][x][co],
+// computes the three taps dy = r - 1 of one dx (r = 3 reads the row below and
+// is not used: three quarters of the rows work).  Three accumulators (dx) of BN
+// columns; K = 16 pixels an MMA.  The bias gradient is summed from the staged
+// dz by the threads that wait.  One stage, two CTAs per SM (one's copies beside
+// the other's MMAs); waits are bounded as in k_conv_tc.
+// Loss and gradient of 64 lattices of 128 x 128: 4430 -> 3949 us (k_wgrad_tc took
+// 227 us for 32 -> 32 channels at 128^2, mostly its 9 x 67 MB of copies).
+__host__ __device__ inline unsigned wgrad_halo_xbytes(int R, int W) { return 64u * (R + 3) * (W + 2); }
+inline size_t wgrad_halo_smem(int R, int W, int BN)
+{
+    return 128 + wgrad_halo_xbytes(R, W) + 2u * BN * R * W + 16;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(kThreads) k_wgrad_halo(ConvSrc S, const bf16 *__restrict__ dz, int H, int W, int Cout,
+                                                         int R, int bands, int per, float *__restrict__ part,
+                                                         float *__restrict__ bias_part)
+{
+    constexpr int BG = BN / 8;
+    constexpr unsigned TCOLS = BN == 32 ? 128 : 256;
+    static_assert(BN == 32 || BN == 64, "three accumulators in at most half the tensor memory");
+    constexpr unsigned IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                               ((unsigned)(BN >> 3) << 17) | ((unsigned)(128 >> 4) << 24);
+    extern __shared__ unsigned char smem_raw[];
+    const unsigned raw = smem_u32(smem_raw);
+    const unsigned sa = (raw + 127u) & ~127u, sb = sa + wgrad_halo_xbytes(R, W);
+    const unsigned bar = sb + 2u * BN * R * W, slot = bar + 8;
+    volatile unsigned *slot_ptr = reinterpret_cast<volatile unsigned *>(smem_raw + (slot - raw));
+
+    const int Cin = S.C0 + S.C1, Wp = W + 2, per_img = H / R;
+    const int cc = blockIdx.x * 32, n0 = blockIdx.y * BN, z = blockIdx.z;
+    const int b0 = z * per, b1 = min(bands, b0 + per);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool first = cc < S.C0, up = first && S.up0, want_bias = bias_part && blockIdx.x == 0;
+    const bf16 *src = first ? S.s0 + cc : S.s1 + (cc - S.C0);
+    const int cs = first ? S.C0 : S.C1, h0 = up ? H >> 1 : H, w0 = up ? W >> 1 : W, sh = up ? 1 : 0;
+    const long long wait_limit = g_tc_wait_limit;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot), "r"(TCOLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = *slot_ptr;
+
+    float bs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    int failed = 0, issued = 0;
+    for (int k = b0; k < b1; ++k) {
+        // the MMAs of the previous band read the buffers this one refills
+        if (k > b0 && !mbar_wait(bar, (k - b0 - 1) & 1, wait_limit)) failed = 1;
+        if (__syncthreads_or(failed)) {
+            failed = 1;
+            break;
+        }
+        const int b = k / per_img, y0 = (k - b * per_img) * R;
+        for (int hy = 0; hy < R + 2; ++hy) {
+            const bf16 *row = src + (size_t)(b * h0 + (wrap(y0 - 1 + hy, H) >> sh)) * w0 * cs;
+            const unsigned d = sa + 64u * hy * Wp;
+            for (int e = tid; e < 4 * W; e += kThreads) {
+                const int x = e >> 2, g = e & 3;
+                cp16(d + 16u * (g * Wp + x + 1), row + (size_t)(x >> sh) * cs + 8 * g);
+            }
+            if (tid < 8) {  // the wrapped columns left and right
+                const int g = tid & 3, x = tid < 4 ? W - 1 : 0;
+                cp16(d + 16u * (g * Wp + (tid < 4 ? 0 : W + 1)), row + (size_t)(x >> sh) * cs + 8 * g);
+            }
+        }
+        for (int y = 0; y < R; ++y) {
+            const bf16 *row = dz + (size_t)((b * H + y0 + y) * W) * Cout + n0;
+            for (int e = tid; e < BG * W; e += kThreads) {
+                const int x = e / BG, c = e % BG;
+                cp16(sb + 16u * ((y * BG + c) * W + x), row + (size_t)x * Cout + 8 * c);
+            }
+        }
+        cp_commit();
+        cp_wait<0>();
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+            tc_fence_after();
+            for (int y = 0; y < R; ++y)
+                for (int x = 0; x < W; x += 16) {
+                    const uint64_t db = desc_ns(sb + 16u * (y * BG * W + x), 128, 16u * W);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+                        tc_mma(tmem + (unsigned)(dx * BN), desc_ns(sa + 16u * (4 * y * Wp + x + dx), 128, 16u * Wp), db,
+                               IDESC, (k > b0 || y > 0 || x > 0) ? 1u : 0u);
+                }
+            tc_commit(bar);
+        }
+        issued = k - b0 + 1;
+        if (want_bias) {
+            const int c = tid % BG;
+            for (int y = 0; y < R; ++y)
+                for (int x = tid / BG; x < W; x += kThreads / BG) {
+                    const uint4 u = *reinterpret_cast<const uint4 *>(smem_raw + (sb - raw) + 16u * ((y * BG + c) * W + x));
+                    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 f = __bfloat1622float2(h[e]);
+                        bs[2 * e] += f.x;
+                        bs[2 * e + 1] += f.y;
+                    }
+                }
+        }
+    }
+    if (issued > 0 && !mbar_wait(bar, (issued - 1) & 1)) failed = 1;
+    failed = __syncthreads_or(failed) || issued < b1 - b0;
+    tc_fence_after();
+    const int q = warp & 3, half = warp >> 2;  // q: dy of the warp's tensor-memory lanes
+    float *pz = part + (size_t)z * Cout * 9 * Cin + cc + lane;
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+        for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 16) {
+            float v[16];
+            tc_ld16(tmem + ((unsigned)(q * 32) << 16) + (unsigned)(dx * BN + c0), v);
+            if (failed || q == 3) continue;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) pz[(size_t)((n0 + c0 + e) * 9 + 3 * q + dx) * Cin] = b1 > b0 ? v[e] : 0.f;
+        }
+    if (want_bias) {  // the block's partial sums of a channel, in order
+        float *red = reinterpret_cast<float *>(smem_raw + (sa - raw));  // [kThreads][8]
+#pragma unroll
+        for (int e = 0; e < 8; ++e) red[8 * tid + e] = bs[e];
+        __syncthreads();
+        if (tid < BN && !failed) {
+            float t = 0.f;
+            for (int p = 0; p < kThreads / BG; ++p) t += red[8 * (p * BG + (tid >> 3)) + (tid & 7)];
+            bias_part[(size_t)z * Cout + n0 + tid] = t;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TCOLS) : "memory");
+    if (failed && tid == 0) atomicExch(&g_tc_error, 1);
+}
+
 // out[i] = sum_{z < nz} part[z * n + i].  A block takes 256 / G values, G
 // threads each: thread g sums z = g, g + G, ... in four running sums (four
 // loads in flight), added as (s0 + s1) + (s2 + s3), and the G sums are added
@@ -1631,11 +1787,36 @@ WgradPlan wgrad_plan(long long P, int Cin, int Cout, bool tc)
     return w;
 }
 
-// workspace for either kernel, so that a workspace sized once stays valid
+// The halo-tile weight gradient: rows of at least kHaloMinWidth pixels (a
+// multiple of the 16 of an MMA), the most of 4, 2, 1 rows per band that divide H
+// and fit two CTAs per SM; R = 0 where it does not apply.  One wave of CTAs.
+struct WgradHalo {
+    int R, bn, bands, per, splits;
+};
+inline int wgrad_halo_bn(int Cout) { return Cout % 64 == 0 ? 64 : 32; }
+inline long long wgrad_halo_splits(int Cin, int Cout)
+{
+    return std::max(1LL, 2LL * 152 / ((Cin / 32) * (Cout / wgrad_halo_bn(Cout))));
+}
+WgradHalo wgrad_halo_plan(int B, int H, int W, int Cin, int Cout)
+{
+    WgradHalo g{0, wgrad_halo_bn(Cout), 0, 0, 0};
+    if (W < kHaloMinWidth || W % 16) return g;
+    for (int R = 4; R >= 1 && !g.R; R /= 2)
+        if (H % R == 0 && wgrad_halo_smem(R, W, g.bn) <= kHaloSmemMax) g.R = R;
+    if (!g.R) return g;
+    g.bands = B * (H / g.R);
+    g.per = (int)((g.bands + wgrad_halo_splits(Cin, Cout) - 1) / wgrad_halo_splits(Cin, Cout));
+    g.splits = (g.bands + g.per - 1) / g.per;
+    return g;
+}
+
+// workspace for any kernel, so that a workspace sized once stays valid
 // when the kernel choice changes
 long long wgrad_ws_bytes(long long P, int Cin, int Cout)
 {
-    long long b = 0;
+    // (the halo tiles' share does not depend on the image's shape)
+    long long b = wgrad_halo_splits(Cin, Cout) * Cout * (9LL * Cin + 1) * (long long)sizeof(float);
     for (int tc = 0; tc < 2; ++tc) {
         WgradPlan w = wgrad_plan(P, Cin, Cout, tc != 0);
         b = std::max(b, (w.part_floats + w.bias_floats) * (long long)sizeof(float));
@@ -1669,11 +1850,38 @@ cudaError_t wgrad_tc_launch(dim3 grid, const ConvSrc &S, const bf16 *dz, int H, 
     return cudaGetLastError();
 }
 
+template <int BN>
+cudaError_t wgrad_halo_launch(const WgradHalo &g, const ConvSrc &S, const bf16 *dz, int H, int Wd, int Cout, float *part,
+                              float *bias_part, cudaStream_t st)
+{
+    static bool attr = false;  // per process; the attribute is per function
+    if (!attr) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_wgrad_halo<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHaloSmemMax);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    const dim3 grid((unsigned)((S.C0 + S.C1) / 32), (unsigned)(Cout / BN), (unsigned)g.splits);
+    k_wgrad_halo<BN><<<grid, kThreads, wgrad_halo_smem(g.R, Wd, BN), st>>>(S, dz, H, Wd, Cout, g.R, g.bands, g.per, part,
+                                                                         bias_part);
+    return cudaGetLastError();
+}
+
 cudaError_t wgrad_launch(const ConvSrc &S, const bf16 *dz, int B, int H, int Wd, int Cout, float *dW, float *db,
                          float *ws, cudaStream_t st)
 {
     long long P = (long long)B * H * Wd;
     int Cin = S.C0 + S.C1;
+    const WgradHalo g = wgrad_halo_plan(B, H, Wd, Cin, Cout);
+    if (g_use_tc == 3 && g.R) {
+        const long long nw = (long long)Cout * 9 * Cin;
+        float *bp = ws + g.splits * nw;
+        cudaError_t e = g.bn == 64 ? wgrad_halo_launch<64>(g, S, dz, H, Wd, Cout, ws, db ? bp : nullptr, st)
+                                   : wgrad_halo_launch<32>(g, S, dz, H, Wd, Cout, ws, db ? bp : nullptr, st);
+        if (e == cudaSuccess) e = sum_parts(ws, g.splits, nw, dW, st);
+        if (e == cudaSuccess && db) e = sum_parts(bp, g.splits, Cout, db, st);
+        return e;
+    }
     WgradPlan w = wgrad_plan(P, Cin, Cout, g_use_tc != 0);
     // the tensor cores sum the bias gradient too where a row tile has a row to
     // spare (and the splits' parts fit the workspace)
