@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kThreads) k_conv_ws(ConvSrc S, const bf16 *__r
 // once per chunk of 32 input channels.  A CTA computes R rows of one image
 // for BN output channels.  Per chunk it stages the band's halo tile -- R + 2
 // rows of W + 2 pixels, the periodic wrap, the upsampling and the channel
-// concatenation resolved through a per-CTA pixel table -- in the no-swizzle
+// concatenation resolved -- in the no-swizzle
 // K-major layout (four planes of 8 channels, 16 bytes per pixel, pixels
 // consecutive) and the chunk's weights of all nine taps.  Outputs are
 // numbered in "slots" with the tile's row pitch W + 2, so that a tap is a
@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(kThreads) k_conv_ws(ConvSrc S, const bf16 *__r
 // with the other's MMAs.  Waits are bounded as in k_conv_tc.
 struct HaloGeom {
     int R, Wp, npix, slots, MT, apix;
-    unsigned a_bytes, b_bytes, tbl_bytes, smem, tcols;
+    unsigned a_bytes, b_bytes, smem, tcols;
 };
 
 constexpr unsigned kHaloSmemMax = 113 * 1024;  // two CTAs per SM
@@ -647,11 +647,15 @@ __host__ __device__ inline HaloGeom halo_geom(int R, int W, int BN)
     g.npix = (R + 2) * g.Wp;
     g.slots = R * g.Wp;
     g.MT = (g.slots + kBM - 1) / kBM;
-    g.apix = g.MT * kBM + 2 * g.Wp + 2;  // the last tile's reads of tap (+1, +1) stay inside
+    // the last tile's slots past the band read up to kBM pixels past a plane:
+    // the next plane, or (16 kBM bytes at most) the weights behind the last
+    // (planes of 2 or 6 pixels modulo 8: the chunks of 4 planes and 2 pixels that a
+    // quarter of a warp copies fall on different banks)
+    g.apix = g.npix;
+    while (g.apix % 8 != 2 && g.apix % 8 != 6) ++g.apix;
     g.a_bytes = 64u * g.apix;
     g.b_bytes = 9u * 64u * BN;
-    g.tbl_bytes = 8u * g.npix;
-    g.smem = 128 + g.a_bytes + g.b_bytes + g.tbl_bytes + 16;
+    g.smem = 128 + g.a_bytes + g.b_bytes + 16;
     unsigned cols = 32;
     while (cols < (unsigned)(g.MT * BN)) cols *= 2;
     g.tcols = cols;
@@ -680,8 +684,7 @@ __global__ void __launch_bounds__(kThreads) k_conv_halo(ConvSrc S, const bf16 *_
     const unsigned raw = smem_u32(smem_raw);
     const unsigned base = (raw + 127u) & ~127u;
     const unsigned sa = base, sb = base + G.a_bytes;
-    int *tbl = reinterpret_cast<int *>(smem_raw + (sb + G.b_bytes - raw));  // [2][npix]
-    const unsigned bar = sb + G.b_bytes + G.tbl_bytes, slot = bar + 8;
+    const unsigned bar = sb + G.b_bytes, slot = bar + 8;
     volatile unsigned *slot_ptr = reinterpret_cast<volatile unsigned *>(smem_raw + (slot - raw));
 
     const int Cin = S.C0 + S.C1, nch = Cin / kBK;
@@ -689,57 +692,59 @@ __global__ void __launch_bounds__(kThreads) k_conv_halo(ConvSrc S, const bf16 *_
     const int n0 = blockIdx.y * BN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long wait_limit = g_tc_wait_limit;
-    // pixel table: source pixel of every tile pixel in src0's grid and in the
-    // full-resolution grid
-    for (int hp = tid; hp < G.npix; hp += kThreads) {
-        const int hy = hp / G.Wp, hx = hp - hy * G.Wp;
-        const int y = wrap(y0 - 1 + hy, H), x = wrap(hx - 1, W);
-        const int full = (b * H + y) * W + x;
-        tbl[hp] = S.up0 ? (b * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1) : full;
-        tbl[G.npix + hp] = full;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot), "r"(G.tcols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
     if (tid == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    tc_fence_before();
-    __syncthreads();  // also publishes the pixel table
-    tc_fence_after();
-    const unsigned tmem = *slot_ptr;
+    unsigned tmem = 0;
     const unsigned lbo_a = 16u * G.apix, lbo_b = 16u * BN;
 
     int failed = 0, issued = 0;
     for (int c = 0; c < nch; ++c) {
         // the MMAs of the previous chunk read the buffers this one refills
-        if (c > 0 && !mbar_wait(bar, (c - 1) & 1, wait_limit)) failed = 1;
-        if (__syncthreads_or(failed)) {
-            failed = 1;
-            break;
+        if (c > 0) {
+            if (!mbar_wait(bar, (c - 1) & 1, wait_limit)) failed = 1;
+            if (__syncthreads_or(failed)) {
+                failed = 1;
+                break;
+            }
         }
         const int cc = c * kBK;
-        const bool first = cc < S.C0;
+        const bool first = cc < S.C0, up = first && S.up0;
         const bf16 *src = first ? S.s0 + cc : S.s1 + (cc - S.C0);
-        const int cs = first ? S.C0 : S.C1;
-        const int *tp = tbl + (first ? 0 : G.npix);
-        for (int e = tid; e < 4 * G.npix; e += kThreads) {
-            const int hp = e >> 2, g = e & 3;
-            cp16(sa + g * lbo_a + 16u * hp, src + (size_t)tp[hp] * cs + g * 8);
+        const int cs = first ? S.C0 : S.C1, sh = up ? 1 : 0;
+        for (int hy = 0; hy < R + 2; ++hy) {
+            const bf16 *row = src + (size_t)(b * (H >> sh) + (wrap(y0 - 1 + hy, H) >> sh)) * (W >> sh) * cs;
+            const unsigned d = sa + 16u * hy * G.Wp;
+            for (int e = tid; e < 4 * W; e += kThreads) {
+                const int x = e >> 2, g = e & 3;
+                cp16(d + g * lbo_a + 16u * (x + 1), row + (size_t)(x >> sh) * cs + 8 * g);
+            }
+            if (tid < 8) {  // the wrapped columns left and right
+                const int g = tid & 3, x = tid < 4 ? W - 1 : 0;
+                cp16(d + g * lbo_a + 16u * (tid < 4 ? 0 : W + 1), row + (size_t)(x >> sh) * cs + 8 * g);
+            }
         }
         for (int e = tid; e < 36 * BN; e += kThreads) {
             const int g = e & 3, nt = e >> 2, n = nt / 9, t = nt - n * 9;
             cp16(sb + (unsigned)(t * 4 + g) * lbo_b + 16u * n, Wk + ((size_t)(n0 + n) * 9 + t) * Cin + cc + g * 8);
         }
         cp_commit();
+        // tensor memory after the first copies are on their way: two CTAs' worth
+        // fits an SM, and a third one waits for it with its tile landing
+        if (c == 0 && warp == 0) {
+            __syncwarp();
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot), "r"(G.tcols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        }
         cp_wait<0>();
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        tc_fence_before();
         __syncthreads();
+        tc_fence_after();
+        tmem = *slot_ptr;
         if (tid == 0) {
-            tc_fence_after();
             for (int mt = 0; mt < G.MT; ++mt)
                 for (int t = 0; t < 9; ++t) {
                     const unsigned a0 = sa + 16u * (unsigned)(mt * kBM + (t / 3) * G.Wp + t % 3);
@@ -1110,10 +1115,14 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_tc(ConvSrc S, const bf16 *__
 // the other's MMAs); waits are bounded as in k_conv_tc.
 // Loss and gradient of 64 lattices of 128 x 128: 4430 -> 3949 us (k_wgrad_tc took
 // 227 us for 32 -> 32 channels at 128^2, mostly its 9 x 67 MB of copies).
+// (a plane of dz has one or two pixels more than a row: the eight 16-byte chunks
+// that a quarter of a warp copies at a time, of 8 planes or of 4 and 2 pixels,
+// fall on different banks)
+__host__ __device__ inline unsigned wgrad_halo_plane(int W, int BN) { return 16u * (W + (BN == 64 ? 1 : 2)); }
 __host__ __device__ inline unsigned wgrad_halo_xbytes(int R, int W) { return 64u * (R + 3) * (W + 2); }
 inline size_t wgrad_halo_smem(int R, int W, int BN)
 {
-    return 128 + wgrad_halo_xbytes(R, W) + 2u * BN * R * W + 16;
+    return 128 + wgrad_halo_xbytes(R, W) + wgrad_halo_plane(W, BN) * (BN / 8) * R + 16;
 }
 
 template <int BN>
@@ -1129,7 +1138,8 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_halo(ConvSrc S, const bf16 *
     extern __shared__ unsigned char smem_raw[];
     const unsigned raw = smem_u32(smem_raw);
     const unsigned sa = (raw + 127u) & ~127u, sb = sa + wgrad_halo_xbytes(R, W);
-    const unsigned bar = sb + 2u * BN * R * W, slot = bar + 8;
+    const unsigned zp = wgrad_halo_plane(W, BN);
+    const unsigned bar = sb + zp * BG * R, slot = bar + 8;
     volatile unsigned *slot_ptr = reinterpret_cast<volatile unsigned *>(smem_raw + (slot - raw));
 
     const int Cin = S.C0 + S.C1, Wp = W + 2, per_img = H / R;
@@ -1180,7 +1190,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_halo(ConvSrc S, const bf16 *
             const bf16 *row = dz + (size_t)((b * H + y0 + y) * W) * Cout + n0;
             for (int e = tid; e < BG * W; e += kThreads) {
                 const int x = e / BG, c = e % BG;
-                cp16(sb + 16u * ((y * BG + c) * W + x), row + (size_t)x * Cout + 8 * c);
+                cp16(sb + zp * (y * BG + c) + 16u * x, row + (size_t)x * Cout + 8 * c);
             }
         }
         cp_commit();
@@ -1191,7 +1201,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_halo(ConvSrc S, const bf16 *
             tc_fence_after();
             for (int y = 0; y < R; ++y)
                 for (int x = 0; x < W; x += 16) {
-                    const uint64_t db = desc_ns(sb + 16u * (y * BG * W + x), 128, 16u * W);
+                    const uint64_t db = desc_ns(sb + zp * (y * BG) + 16u * x, 128, zp);
 #pragma unroll
                     for (int dx = 0; dx < 3; ++dx)
                         tc_mma(tmem + (unsigned)(dx * BN), desc_ns(sa + 16u * (4 * y * Wp + x + dx), 128, 16u * Wp), db,
@@ -1204,7 +1214,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_halo(ConvSrc S, const bf16 *
             const int c = tid % BG;
             for (int y = 0; y < R; ++y)
                 for (int x = tid / BG; x < W; x += kThreads / BG) {
-                    const uint4 u = *reinterpret_cast<const uint4 *>(smem_raw + (sb - raw) + 16u * ((y * BG + c) * W + x));
+                    const uint4 u = *reinterpret_cast<const uint4 *>(smem_raw + (sb - raw) + zp * (y * BG + c) + 16u * x);
                     const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -1788,8 +1798,10 @@ WgradPlan wgrad_plan(long long P, int Cin, int Cout, bool tc)
 }
 
 // The halo-tile weight gradient: rows of at least kHaloMinWidth pixels (a
-// multiple of the 16 of an MMA), the most of 4, 2, 1 rows per band that divide H
-// and fit two CTAs per SM; R = 0 where it does not apply.  One wave of CTAs.
+// multiple of the 16 of an MMA; rows of 32 pixels: 3902 -> 3959 us for the loss and
+// gradient of 64 lattices of 128 x 128), the most of 8, 4, 2, 1 rows per band that
+// divide H, hold at most 512 pixels (256: 4124 us) and fit two CTAs per SM; R = 0
+// where it does not apply.  One wave of CTAs.
 struct WgradHalo {
     int R, bn, bands, per, splits;
 };
@@ -1802,8 +1814,8 @@ WgradHalo wgrad_halo_plan(int B, int H, int W, int Cin, int Cout)
 {
     WgradHalo g{0, wgrad_halo_bn(Cout), 0, 0, 0};
     if (W < kHaloMinWidth || W % 16) return g;
-    for (int R = 4; R >= 1 && !g.R; R /= 2)
-        if (H % R == 0 && wgrad_halo_smem(R, W, g.bn) <= kHaloSmemMax) g.R = R;
+    for (int R = 8; R >= 1 && !g.R; R /= 2)
+        if (H % R == 0 && R * W <= 512 && wgrad_halo_smem(R, W, g.bn) <= kHaloSmemMax) g.R = R;
     if (!g.R) return g;
     g.bands = B * (H / g.R);
     g.per = (int)((g.bands + wgrad_halo_splits(Cin, Cout) - 1) / wgrad_halo_splits(Cin, Cout));

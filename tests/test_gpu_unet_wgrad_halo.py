@@ -71,10 +71,10 @@ def test_weight_gradient_on_halo_tiles(case):
 
 
 def test_a_wait_that_runs_out_is_reported():
-    # 32 bands over 25 splits: some CTA waits for its first band's MMAs
+    # 32 bands of 8 rows over 25 splits: some CTA waits for its first band's MMAs
     rng = np.random.default_rng(3)
-    s0, x0 = rand_bf(rng, (2, 64, 64, 128))
-    dzt, dz = rand_bf(rng, (2, 64, 64, 96))
+    s0, x0 = rand_bf(rng, (4, 64, 64, 128))
+    dzt, dz = rand_bf(rng, (4, 64, 64, 96))
     try:
         UN.set_wait_limit(0)
         UN.conv3x3_wgrad(s0, dzt)
