@@ -87,6 +87,21 @@ __device__ __forceinline__ v3<double> ld(const dq4 *p, long i)
     double2 a = __ldg(q), b = __ldg(q + 1);
     return {a.x, a.y, b.x};
 }
+// L2 loads for what the kernel just before wrote.  A kernel launched with
+// programmatic serialisation runs beside it until wait_prerequisite(), and a
+// load through the read-only path (__ldg) is one of constant memory to the
+// compiler, which may move it above that wait.
+__device__ __forceinline__ v3<float> ldl2(const float4 *p, long i)
+{
+    float4 v = __ldcg(p + i);
+    return {v.x, v.y, v.z};
+}
+__device__ __forceinline__ v3<double> ldl2(const dq4 *p, long i)
+{
+    const double2 *q = reinterpret_cast<const double2 *>(p + i);
+    double2 a = __ldcg(q), b = __ldcg(q + 1);
+    return {a.x, a.y, b.x};
+}
 // plain (coherent) loads for buffers written earlier in the same kernel
 __device__ __forceinline__ v3<float> ldc(const float4 *p, long i)
 {
@@ -451,6 +466,16 @@ __device__ __forceinline__ v3<float> local_field_comp(const Stencil<float> &S, c
 // the launch attribute both are no-ops.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisite() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// The same, and the compiler takes the pointers for new ones after it: loads
+// through the read-only path (__ldg, const __restrict__) are loads of constant
+// memory to it, which a memory clobber does not hold back, and 20 steps of a film
+// with dipoles came out differently from run to run.
+template <typename P> __device__ __forceinline__ void renew(P &p) { asm volatile("" : "+l"(p)); }
+template <typename... P> __device__ __forceinline__ void wait_prerequisite(P &...p)
+{
+    wait_prerequisite();
+    (renew(p), ...);
+}
 
 // Launch a kernel that calls wait_prerequisite() before it reads anything
 // written earlier on the stream, with programmatic stream serialisation --

@@ -340,7 +340,7 @@ __device__ __forceinline__ void segment(const CubicParams<T> &P, const rec_t<T> 
             qa[j][k] = mk(T(0), T(0), T(0));
             if (PASS == 1 && SOLVER != SP_RK4 && !QS && own[j] && za + k < zb) qa[j][k] = ld(q, i[j] + k * plane_sz);
         }
-        if (HAS_BDD && own[j]) bn[j] = ld(Bdd, i[j]);
+        if (HAS_BDD && own[j]) bn[j] = ldl2(Bdd, i[j]);
     }
     int s_next = 2 % NB, s_free = 1;  // slots of planes z+1 and z
     const uint64_t step = REPL && (PASS == 0 || SOLVER == SP_RK4) ? llg_step_of(c) : c.step;  // Philox step
@@ -357,7 +357,7 @@ __device__ __forceinline__ void segment(const CubicParams<T> &P, const rec_t<T> 
             for (int k = 0; k + 1 < QA; ++k) qa[j][k] = qa[j][k + 1];
             if (own[j] && z + QA < zb && PASS == 1 && SOLVER != SP_RK4 && !QS)
                 qa[j][QA - 1] = ld(q, i[j] + QA * plane_sz);
-            if (HAS_BDD && own[j] && z + 1 < zb) bn[j] = ld(Bdd, i[j] + plane_sz);
+            if (HAS_BDD && own[j] && z + 1 < zb) bn[j] = ldl2(Bdd, i[j] + plane_sz);
         }
         cp_async_wait<NB - 2>();
         __syncthreads();
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(TX *TY, (MinBlocks<SOLVER, PASS, ROWS>::value)
     __shared__ __align__(32) rec_t<T> tiles[NB][Tile<ROWS>::HN];
     __shared__ __align__(32) rec_t<T> qtiles[QS ? NB : 1][QS ? TX * TY * ROWS : 1];
     allow_dependents();
-    wait_prerequisite();  // the previous pass reads what this one overwrites
+    wait_prerequisite(src, np, q, nout, Bdd);  // the previous pass reads what this one overwrites
     int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + Tile<ROWS>::TYE - 1) / Tile<ROWS>::TYE;
     long ntile = (long)tiles_x * tiles_y;
     long total = ntile * P.nz * (REPL ? llg_reps(c) : 1);

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
 #pragma unroll
     for (int n2 = 0; n2 < 16; ++n2) {  // x < 512: the upper half is padding
         int x = 32 * n2 + lane;
-        float4 v = (row && x < n0) ? __ldg(&n[(long)y * n0 + x]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 v = (row && x < n0) ? __ldcg(&n[(long)y * n0 + x]) : make_float4(0.f, 0.f, 0.f, 0.f);
         a[n2] = part ? make_float2(v.x, v.y) : make_float2(v.z, 0.f);
         a[n2 + 16] = make_float2(0.f, 0.f);
     }

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kBlock) k_field(const __grid_constant__ Stenci
     int b;
     v3<T> ni = ld(n, i);
     v3<T> B = local_field(S, n, i, ni, b);
-    if (Bdd) B = B + ld(Bdd, i);
+    if (Bdd) B = B + ldl2(Bdd, i);
     st(out, i, sign * B);
 }
 
@@ -67,7 +67,7 @@ __device__ __forceinline__ void pred_spin(const Stencil<T> &S, const R *n, const
     int b;
     v3<T> ni = ld(n, i);
     v3<T> B = local_field(S, n, i, ni, b);
-    if (Bdd) B = B + ld(Bdd, i);
+    if (Bdd) B = B + ldl2(Bdd, i);
     v3<T> Bth = mk(T(0), T(0), T(0));
     if (c.thermal) Bth = noise_amp(c, r, b) * box_muller(thermal_bits(c, (uint32_t)i, (uint32_t)r), T(0));
     v3<T> A = llg_A(c.cA[b], c.alpha, ni, B + Bth);
@@ -96,7 +96,7 @@ __device__ __forceinline__ void corr_spin(const Stencil<T> &S, R *n, const R *np
     int b;
     v3<T> p = ld(np, i);
     v3<T> B = local_field(S, np, i, p, b);
-    if (Bdd) B = B + ld(Bdd, i);
+    if (Bdd) B = B + ldl2(Bdd, i);
     v3<T> Ap = llg_A(c.cA[b], c.alpha, p, B);
     v3<T> qi = ld(q, i);
     if (SOLVER == SP_HEUN) {
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_
                                                      rec_t<T> *__restrict__ q, const LlgConst<T> c)
 {
     allow_dependents();
-    wait_prerequisite();  // n (and Bdd) come from the kernels before
+    wait_prerequisite(n, Bdd);  // they come from the kernels before
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S.N) return;
     int r = blockIdx.y;  // replica
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_
                                                      const rec_t<T> *__restrict__ Bdd, const LlgConst<T> c)
 {
     allow_dependents();
-    wait_prerequisite();  // np, q (and Bdd) come from the kernels before
+    wait_prerequisite(n, np, q, Bdd);  // they come from the kernels before
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S.N) return;
     size_t o = (size_t)blockIdx.y * S.N;  // replica
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kBlock) k_llg_bpred(const int2 *__restrict__ b
                                                       const LlgConst<T> c)
 {
     allow_dependents();
-    wait_prerequisite();  // n comes from the kernels before
+    wait_prerequisite(n);  // it comes from the kernels before
     const int2 bt = blk[blockIdx.x];
     const LlgConst<T> &cs = batch_const(c, sys[bt.x]);
     const Stencil<T> &S = Sv[bt.x];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kBlock) k_llg_bcorr(const int2 *__restrict__ b
                                                       const LlgConst<T> c)
 {
     allow_dependents();
-    wait_prerequisite();  // np, q come from the kernels before
+    wait_prerequisite(n, np, q);  // they come from the kernels before
     const int2 bt = blk[blockIdx.x];
     const LlgConst<T> &cs = batch_const(c, sys[bt.x]);
     const Stencil<T> &S = Sv[bt.x];
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kBlock) k_rk4(const __grid_constant__ Stencil<
                                                 const LlgConst<T> c)
 {
     allow_dependents();
-    wait_prerequisite();  // the stage inputs come from the kernels before
+    wait_prerequisite(n, src, acc, Bdd);  // the stage inputs come from the kernels before
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S.N) return;
     int r = blockIdx.y;  // replica
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kBlock) k_rk4(const __grid_constant__ Stencil<
     int b;
     v3<T> y = ld(src, i);
     v3<T> B = local_field(S, src, i, y, b);
-    if (Bdd) B = B + ld(Bdd, i);
+    if (Bdd) B = B + ldl2(Bdd, i);
     if (c.thermal) B = B + noise_amp(c, r, b) * box_muller(thermal_bits(c, (uint32_t)i, (uint32_t)r), T(0));
     v3<T> k = cross(y, llg_A(c.cA[b], c.alpha, y, B));
     v3<T> ni = ldc(n, i);
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kBlock) k_energy(const __grid_constant__ Stenc
         acc[4] = -0.5 * ddot(ni, Bd);
         B = B + Bx + Bd;
         if (Bdd) {
-            v3<T> bd = ld(Bdd, i);
+            v3<T> bd = ldl2(Bdd, i);
             acc[5] = -0.5 * ddot(ni, bd);
             B = B + bd;
         }

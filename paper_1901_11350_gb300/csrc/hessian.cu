@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kHB) k_hvp(const __grid_constant__ Stencil<T> 
                                              unsigned *status = nullptr)
 {
     allow_dependents();
-    wait_prerequisite();  // n and v may come from the kernels before
+    wait_prerequisite(n, v);  // they may come from the kernels before
     int i = blockIdx.x * kHB + threadIdx.x;
     if (i >= S.N) return;
     int b, c0, c1, c2;

@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_v
                                                      const int *state)
 {
     allow_dependents();
-    wait_prerequisite();  // state, scalars and records come from the kernels before
+    wait_prerequisite(x, v, F, scal, state);  // state, scalars and records come from the kernels before
     if (mode && state[1] == 0) return;
     const int i = blockIdx.x * kBlock + threadIdx.x;
     const T c = mode == 2 ? (T)scal[kC] : T(0);
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kBlock) k_vp_move(int N, rec_t<T> *__restrict_
                                                     int k, int max_iter, const double *scal, int *state)
 {
     allow_dependents();
-    wait_prerequisite();  // state, scalars and records come from the kernels before
+    wait_prerequisite(x, v, F, scal, state);  // state, scalars and records come from the kernels before
     const bool done = scal[kFN] < tol || k >= max_iter;
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i < N) vp_move(x, v, F, i, dt, dt2_2m, scal[kVP] != 0.0, (T)scal[kC], done, k >= max_iter);
@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_b
     Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
     stage_stencil(S + bi.chain, &St);
     allow_dependents();
-    wait_prerequisite();  // state, scalars and records come from the kernels before
+    wait_prerequisite(x, v, F, scal, state);  // state, scalars and records come from the kernels before
     if (mode && state[2 * bi.g + 1] == 0) return;
     double *sc = scal + kS * bi.g;
     const T c = mode == 2 ? (T)sc[kC] : T(0);
@@ -925,7 +925,7 @@ __global__ void __launch_bounds__(kBlock) k_bvp_move(const BlkInfo *__restrict__
     const BlkInfo bi = blk[blockIdx.x];
     const ImgInfo im = img[bi.g];
     allow_dependents();
-    wait_prerequisite();  // state, scalars and records come from the kernels before
+    wait_prerequisite(x, v, F, scal, state, proj);  // state, scalars and records come from the kernels before
     const double *sc = scal + kS * bi.g;
     const bool done = sc[kFN] < tol || k >= max_iter;
     const int i = bi.t * kBlock + threadIdx.x;

@@ -83,3 +83,25 @@ def test_a_wait_that_runs_out_is_reported():
         UN.set_wait_limit()
     _check(s0, x0, dzt, dz)
     assert UN.lib().sp_unet_device_error() == 0
+
+
+@pytest.mark.parametrize("shape", [(1, 64, 64, 32, 32), (1, 8, 128, 32, 64), (2, 16, 16, 32, 128)])
+def test_outputs_and_masks_on_16_byte_boundaries(shape):
+    # 32-byte rows at once where out and mask allow it, two 16-byte ones elsewhere
+    B, H, W, Cin, Cout = shape
+    rng = np.random.default_rng(9)
+    x, _ = rand_bf(rng, (B, H, W, Cin))
+    Wt, _ = rand_bf(rng, (Cout, 9, Cin))
+    mask, _ = rand_bf(rng, (B, H, W, Cout))
+    want = UN.conv3x3_forward(x, Wt, None, relu=False, mask=mask)
+    n = want.numel()
+    for mo, oo in ((0, 8), (8, 0), (8, 8)):
+        m = torch.zeros(n + 16, dtype=torch.bfloat16, device="cuda")
+        out = torch.full((n + 16,), 7.0, dtype=torch.bfloat16, device="cuda")
+        m[mo:mo + n] = mask.reshape(-1)
+        rc = UN.lib().sp_conv3x3_forward(x.data_ptr(), Cin, 0, None, 0, Wt.data_ptr(), None, 0, m.data_ptr() + 2 * mo, B,
+                                         H, W, Cout, out.data_ptr() + 2 * oo, torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+        assert torch.equal(out[oo:oo + n], want.reshape(-1))
+        assert bool(torch.all(out[:oo] == 7.0)) and bool(torch.all(out[oo + n:] == 7.0))
+    UN.check_device_error()
