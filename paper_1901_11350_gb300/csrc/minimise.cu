@@ -152,7 +152,6 @@ __device__ __forceinline__ f2sum acc_dot(v3<float> a, v3<float> b)
 {
     return acc_prod(a.x, b.x) + acc_prod(a.y, b.y) + acc_prod(a.z, b.z);
 }
-__device__ __forceinline__ double acc_prod(double a, double b) { return __dmul_rn(a, b); }
 // r += a.b for a sum of a few spins: the products and the errors of the
 // additions to r.hi go to r.lo one after another
 __device__ __forceinline__ void acc_add(f2sum &r, float a, float b)
