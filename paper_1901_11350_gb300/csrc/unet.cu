@@ -1801,19 +1801,28 @@ struct WgradPlan {
 
 int wgrad_tc_bn(int Cout) { return Cout % 256 == 0 ? 256 : (Cout % 128 == 0 ? 128 : (Cout % 64 == 0 ? 64 : 32)); }
 
-// Pixel splits: enough CTAs for a few per SM over the tiles; each split a
-// whole number of 32-pixel steps.
+// Pixel splits wanted: enough CTAs for a few per SM over the tiles (tcgen05: one
+// wave of CTAs at the occupancy the stages' shared memory allows; fewer splits
+// also mean fewer partial sums to add up).
+long long wgrad_splits_wanted(int Cin, int Cout, bool tc)
+{
+    if (!tc) {
+        const long long base = (long long)(Cout / (Cout % 64 == 0 ? 64 : 32)) * 9 * (Cin / kBK);
+        return (4LL * 152 + base - 1) / base;
+    }
+    const int bn = wgrad_tc_bn(Cout);
+    const long long base = ((9LL * Cin + 127) / 128) * (Cout / bn);
+    return std::max(1LL, 152LL * (bn == 256 ? 2 : (bn == 128 ? 3 : (bn == 64 ? 4 : 5))) / base);
+}
+
+// The splits: as many as wanted, each a whole number of 32-pixel steps.
 WgradPlan wgrad_plan(long long P, int Cin, int Cout, bool tc)
 {
     WgradPlan w;
     w.bmc = Cout % 64 == 0 ? 64 : 32;
     w.tc_bn = tc ? wgrad_tc_bn(Cout) : 0;
-    long long base = tc ? ((9LL * Cin + 127) / 128) * (Cout / w.tc_bn) : (long long)(Cout / w.bmc) * 9 * (Cin / kBK);
     long long chunks = P / 32;
-    // tcgen05: one wave of CTAs at the occupancy the stages' shared memory
-    // allows (fewer splits also mean fewer partial sums to add up)
-    const long long res = !tc ? 4 : (w.tc_bn == 256 ? 2 : (w.tc_bn == 128 ? 3 : (w.tc_bn == 64 ? 4 : 5)));
-    long long s = tc ? std::max(1LL, 152 * res / base) : (4LL * 152 + base - 1) / base;
+    long long s = wgrad_splits_wanted(Cin, Cout, tc);
     if (s > chunks) s = chunks;
     if (s < 1) s = 1;
     long long per = (chunks + s - 1) / s;
@@ -1865,6 +1874,21 @@ long long wgrad_ws_bytes(long long P, int Cin, int Cout)
         b = std::max(b, (w.part_floats + w.bias_floats) * (long long)sizeof(float));
     }
     return b;
+}
+
+// Workspace bytes that hold the partials of every batch of at most P pixels.
+// The splits of a smaller batch can be more than those of P itself (whole steps
+// per split: 61 chunks in 41 splits wanted make 31 splits, 41 chunks make 41), so
+// the bound takes the splits that are wanted, which grow with the pixels.
+long long wgrad_ws_bound(long long P, int Cin, int Cout)
+{
+    long long b = 0;
+    for (int tc = 0; tc < 2; ++tc) {
+        const long long s = std::max(1LL, std::min(wgrad_splits_wanted(Cin, Cout, tc != 0), P / 32));
+        const long long bias = std::min(2LL * 152, (P + 1023) / 1024);
+        b = std::max(b, (s * 9 * Cin + bias) * Cout * (long long)sizeof(float));
+    }
+    return std::max(b, wgrad_halo_splits(Cin, Cout) * Cout * (9LL * Cin + 1) * (long long)sizeof(float));
 }
 
 // Eight threads per value from 32 partials on: below, the loads of one thread
@@ -2170,7 +2194,7 @@ int sp_unet_create(sp_unet **out, int L, int batch_max)
     long long ws = 0;
     for (int l = 0; l < SP_UNET_LAYERS; ++l) {
         long long P = level_pixels(n, batch_max, kLayers[l].level);
-        long long b = wgrad_ws_bytes(P, n->tab.cin[l], kLayers[l].cout) / (long long)sizeof(float);
+        long long b = wgrad_ws_bound(P, n->tab.cin[l], kLayers[l].cout) / (long long)sizeof(float);
         if (b > ws) ws = b;
     }
     n->ws_floats = ws;
