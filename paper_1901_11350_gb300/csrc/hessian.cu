@@ -630,7 +630,7 @@ struct Ops {
     // Lowest eigenpair of H at n by m Lanczos steps from `start` (allow_seed:
     // a zero start selects a fixed pseudo-random tangent field).  mode
     // receives the unit Ritz vector.  One synchronisation, for the
-    // tridiagonal matrix.
+    // tridiagonal matrix: on return the launches that form the mode are queued.
     int lowest(const rec_t<T> *n, const rec_t<T> *start, bool allow_seed, rec_t<T> *mode, int m, double *lam)
     {
         // the Krylov space cannot outgrow the 2N-dimensional tangent space
@@ -727,7 +727,10 @@ int lowest_mode_run(sp_ctx *c, const Stencil<T> &S, const void *n, void *mode, i
     if (rc) return rc;
     Ops<T> op{S, *c->hess, st, c->N, hblocks(c->N)};
     rec_t<T> *md = (rec_t<T> *)mode;
-    return op.lowest((const rec_t<T> *)n, md, true, md, m, lam);
+    if ((rc = op.lowest((const rec_t<T> *)n, md, true, md, m, lam))) return rc;
+    // the launches that form the mode read the context's scratch, and the next
+    // call may come on another stream
+    return cudaStreamSynchronize(st) == cudaSuccess ? 0 : SP_ERR_CUDA;
 }
 
 template <typename T>
