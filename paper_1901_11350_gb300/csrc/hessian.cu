@@ -244,40 +244,60 @@ template <typename T> __device__ __forceinline__ v3<T> seed_field(int i)
     return mk((T)((int)(h[0] >> 8) - (1 << 23)), (T)((int)(h[1] >> 8) - (1 << 23)), (T)((int)(h[2] >> 8) - (1 << 23)));
 }
 
-// part[block] = partial of |v|^2
-template <typename T> __global__ void __launch_bounds__(kLzB) k_lz_norm(int N, const rec_t<T> *v, double *part)
+// part[block] = the largest |component| of v in the block's share (NaN if one
+// is).  The start vector is scaled by a power of two near its inverse before
+// anything is squared: a start of any size gives the bits of a start of unit
+// size, also where squares of FP32 records would under- or overflow.
+template <typename T> __global__ void __launch_bounds__(kLzB) k_lz_size(int N, const rec_t<T> *v, double *part)
 {
+    __shared__ T sh[kLzB / 32];
     wait_prerequisite();
-    typename LzAcc<T>::type s{};
+    T m = 0;
     for (int i = blockIdx.x * kLzB + threadIdx.x; i < N; i += gridDim.x * kLzB) {
         const v3<T> a = ldc(v, i);
-        s = s + lz_dot(a, a);
+        m = nan_max(m, nan_max(fabs(a.x), nan_max(fabs(a.y), fabs(a.z))));
     }
     allow_dependents();
-    const double r = block_sum(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = r;
+    for (int o = 16; o > 0; o >>= 1) m = nan_max(m, shfl_down(m, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kLzB / 32; ++w) m = nan_max(m, sh[w]);
+        part[blockIdx.x] = (double)m;
+    }
 }
 
-// w = start projected onto the tangent planes of n (a zero start, by its nN
-// norm partials startN: the fixed pseudo-random field where allow_seed), partN
-// its norm, nB_i = n_i . B_i (the Weingarten term of every product of the run).
+// w = start, scaled, projected onto the tangent planes of n (a zero start, by
+// the nS partials startS of its size: the fixed pseudo-random field where
+// allow_seed), partN its norm, nB_i = n_i . B_i (the Weingarten term of every
+// product of the run).
 template <typename T>
 __global__ void __launch_bounds__(kLzB) k_lz_begin(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ n,
-                                                   const rec_t<T> *start, int allow_seed, const double *startN, int nN,
+                                                   const rec_t<T> *start, int allow_seed, const double *startS, int nS,
                                                    rec_t<T> *w, T *nB, double *partN)
 {
     __shared__ int s_seed;
+    __shared__ T s_scale[2];
     wait_prerequisite();
     if (threadIdx.x < 32) {
-        const double z = partial_sum(startN, nN);
-        if (threadIdx.x == 0) s_seed = allow_seed && !(z > 0);
+        double z = 0;
+        for (int p = threadIdx.x; p < nS; p += 32) z = nan_max(z, __ldcg(startS + p));
+        for (int o = 16; o > 0; o >>= 1) z = nan_max(z, lz_xor(z, o));
+        if (threadIdx.x == 0) {
+            s_seed = allow_seed && !(z > 0);
+            // in two factors: 2^-e alone can be out of T's range
+            const int e = z > 0 && isfinite(z) ? ilogb(z) : 0;
+            s_scale[0] = (T)scalbn(1.0, -(e / 2));
+            s_scale[1] = (T)scalbn(1.0, -(e - e / 2));
+        }
     }
     __syncthreads();
     const bool seed = s_seed;
+    const T s0 = s_scale[0], s1 = s_scale[1];
     typename LzAcc<T>::type s{};
     for (int i = blockIdx.x * kLzB + threadIdx.x; i < S.N; i += gridDim.x * kLzB) {
         int b;
-        const v3<T> ni = ldc(n, i), vi = seed ? seed_field<T>(i) : ldc(start, i);
+        const v3<T> ni = ldc(n, i), vi = seed ? seed_field<T>(i) : s1 * (s0 * ldc(start, i));
         const v3<T> wi = vi - dot(vi, ni) * ni;
         st(w, i, wi);
         nB[i] = dot(ni, local_field(S, n, i, ni, b));
@@ -324,7 +344,7 @@ __global__ void __launch_bounds__(kLzB) k_lz_apply(const __grid_constant__ Stenc
             double tnorm = 0;
             if (k > 0) tnorm = fabs(run->alpha[k - 1]) + b;
             if (k > 1) tnorm = fmax(run->tnorm[k - 1], tnorm + run->beta[k - 2]);
-            const bool go = k ? b > brk * tnorm : b2 > 0;
+            const bool go = k ? b > brk * tnorm : b2 > 0 && isfinite(b2);
             s_inv = go ? 1.0 / b : 0.0;
             if (blockIdx.x == 0) {
                 if (go) {
@@ -332,7 +352,7 @@ __global__ void __launch_bounds__(kLzB) k_lz_apply(const __grid_constant__ Stenc
                     run->tnorm[k] = tnorm;
                     if (k) run->beta[k - 1] = b;
                 } else if (k == 0) {
-                    run->nan_start = b2 != b2;
+                    run->nan_start = !isfinite(b2);
                 }
             }
         }
@@ -645,7 +665,7 @@ struct Ops {
         if (cudaMemsetAsync(run, 0, sizeof(LzRun), st) != cudaSuccess) return SP_ERR_CUDA;
         // launched plainly: all that was written before the run is in place
         // before any kernel of the run begins
-        k_lz_norm<T><<<gs, bs, 0, st>>>(N, start, pA);
+        k_lz_size<T><<<gs, bs, 0, st>>>(N, start, pA);
         cudaError_t e = launch_pdl(k_lz_begin<T>, gs, bs, 0, st, S, n, start, (int)allow_seed, (const double *)pA, nS,
                                    W[0], nB, pN);
         for (int k = 0; k < m && e == cudaSuccess; ++k) {

@@ -46,3 +46,27 @@ def test_two_streams_give_the_modes_of_single_calls(prec):
         torch.cuda.synchronize()
         for (lam, m), (l0, m0) in zip(out, single):
             assert lam == l0 and torch.equal(m, m0)
+
+
+@pytest.mark.parametrize("prec,exponents", [("f32", (-100, -80, 70, 120)), ("f64", (-900, -600, 550, 1000))])
+def test_start_vectors_of_any_size(prec, exponents):
+    # a power of two changes no rounding of the run: the same bits
+    c, (n, _), v = _system(40, prec)
+    lam, mode = c.lowest_mode(n, v.clone(), 24)
+    seeded = c.lowest_mode(n, torch.zeros_like(v), 24)[1]
+    assert not torch.equal(mode, seeded)
+    for e in exponents:
+        l2, m2 = c.lowest_mode(n, v * 2.0 ** e, 24)
+        assert l2 == lam and torch.equal(m2, mode), e
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_start_vector_that_is_not_finite(prec):
+    # infinite: reported; NaN: replaced, as a zero one is
+    c, (n, _), v = _system(40, prec)
+    w = v.clone()
+    w[7, 1] = float("inf")
+    with pytest.raises(B.SpinError):
+        c.lowest_mode(n, w, 8)
+    w[7, 1] = float("nan")
+    assert torch.equal(c.lowest_mode(n, w, 8)[1], c.lowest_mode(n, torch.zeros_like(v), 8)[1])
