@@ -143,7 +143,10 @@ int sp_unet_device_error(void);
  * warp-specialised kernel (2) keeps the default limit. */
 int sp_conv3x3_set_wait_limit(long long cycles);
 
-/* Workspace bytes sp_conv3x3_wgrad needs for this shape. */
+/* Workspace bytes sp_conv3x3_wgrad needs for this shape, whichever kernel is
+ * chosen.  Kernel 3 needs more than the others for rows it takes (at least 64
+ * pixels); with a workspace that suffices for those alone it leaves the call
+ * to kernel 1. */
 long long sp_conv3x3_wgrad_workspace(int B, int H, int Wd, int Cin, int Cout);
 
 /* Weight gradient dW[co][t][ci] = sum_p dz[p][co] * in_t[p][ci] (FP32) and,

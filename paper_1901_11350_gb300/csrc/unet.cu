@@ -1863,17 +1863,29 @@ WgradHalo wgrad_halo_plan(int B, int H, int W, int Cin, int Cout)
     return g;
 }
 
-// workspace for any kernel, so that a workspace sized once stays valid
-// when the kernel choice changes
-long long wgrad_ws_bytes(long long P, int Cin, int Cout)
+// Bytes of the halo tiles' partials; 0 where they do not apply.
+long long wgrad_halo_bytes(const WgradHalo &g, int Cin, int Cout)
 {
-    // (the halo tiles' share does not depend on the image's shape)
-    long long b = wgrad_halo_splits(Cin, Cout) * Cout * (9LL * Cin + 1) * (long long)sizeof(float);
+    return g.R ? (long long)g.splits * Cout * (9LL * Cin + 1) * (long long)sizeof(float) : 0;
+}
+
+// Workspace that kernels 0 to 2 need, whichever is chosen: the least a call takes.
+long long wgrad_least_bytes(long long P, int Cin, int Cout)
+{
+    long long b = 0;
     for (int tc = 0; tc < 2; ++tc) {
         WgradPlan w = wgrad_plan(P, Cin, Cout, tc != 0);
         b = std::max(b, (w.part_floats + w.bias_floats) * (long long)sizeof(float));
     }
     return b;
+}
+
+// Workspace for any kernel, so that a workspace sized once stays valid
+// when the kernel choice changes.
+long long wgrad_ws_bytes(int B, int H, int W, int Cin, int Cout)
+{
+    return std::max(wgrad_least_bytes((long long)B * H * W, Cin, Cout),
+                    wgrad_halo_bytes(wgrad_halo_plan(B, H, W, Cin, Cout), Cin, Cout));
 }
 
 // Workspace bytes that hold the partials of every batch of at most P pixels.
@@ -1935,12 +1947,12 @@ cudaError_t wgrad_halo_launch(const WgradHalo &g, const ConvSrc &S, const bf16 *
 }
 
 cudaError_t wgrad_launch(const ConvSrc &S, const bf16 *dz, int B, int H, int Wd, int Cout, float *dW, float *db,
-                         float *ws, cudaStream_t st)
+                         float *ws, long long ws_bytes, cudaStream_t st)
 {
     long long P = (long long)B * H * Wd;
     int Cin = S.C0 + S.C1;
     const WgradHalo g = wgrad_halo_plan(B, H, Wd, Cin, Cout);
-    if (g_use_tc == 3 && g.R) {
+    if (g_use_tc == 3 && g.R && wgrad_halo_bytes(g, Cin, Cout) <= ws_bytes) {
         const long long nw = (long long)Cout * 9 * Cin;
         float *bp = ws + g.splits * nw;
         cudaError_t e = g.bn == 64 ? wgrad_halo_launch<64>(g, S, dz, H, Wd, Cout, ws, db ? bp : nullptr, st)
@@ -2109,7 +2121,7 @@ cudaError_t backward(sp_unet *n, int batch, cudaStream_t st)
         int s = L >> d.level;
         ConvSrc S = layer_src(n, l);
         cudaError_t e = wgrad_launch(S, n->dz[l], batch, s, s, d.cout, n->grad + n->off.w[l], n->grad + n->off.b[l],
-                                     n->ws, st);
+                                     n->ws, n->ws_floats * (long long)sizeof(float), st);
         if (e != cudaSuccess) return e;
         if (l == 0) break;
         int cin = d.cin0 + d.cin1;
@@ -2378,7 +2390,7 @@ int sp_unet_device_error(void)
 long long sp_conv3x3_wgrad_workspace(int B, int H, int Wd, int Cin, int Cout)
 {
     if (B < 1 || H < 1 || Wd < 1 || Cin < 32 || Cout < 32) return -1;
-    return wgrad_ws_bytes((long long)B * H * Wd, Cin, Cout);
+    return wgrad_ws_bytes(B, H, Wd, Cin, Cout);
 }
 
 int sp_conv3x3_wgrad(const uint16_t *src0, int C0, int up0, const uint16_t *src1, int C1, const uint16_t *dz, int B,
@@ -2387,9 +2399,10 @@ int sp_conv3x3_wgrad(const uint16_t *src0, int C0, int up0, const uint16_t *src1
 {
     if (!src0 || !dz || !dW || !workspace || (C1 && !src1)) return SP_ERR_ARG;
     if (!conv_shape_ok(C0, C1, up0, B, H, Wd, Cout)) return SP_ERR_ARG;
-    if (workspace_bytes < wgrad_ws_bytes((long long)B * H * Wd, C0 + C1, Cout)) return SP_ERR_ARG;
+    if (workspace_bytes < wgrad_least_bytes((long long)B * H * Wd, C0 + C1, Cout)) return SP_ERR_ARG;
     ConvSrc S{(const bf16 *)src0, C0, up0 ? 1 : 0, (const bf16 *)src1, C1};
-    cudaError_t e = wgrad_launch(S, (const bf16 *)dz, B, H, Wd, Cout, dW, db, (float *)workspace, (cudaStream_t)stream);
+    cudaError_t e = wgrad_launch(S, (const bf16 *)dz, B, H, Wd, Cout, dW, db, (float *)workspace, workspace_bytes,
+                                 (cudaStream_t)stream);
     return e == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 
