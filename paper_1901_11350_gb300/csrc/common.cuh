@@ -376,13 +376,20 @@ __device__ __forceinline__ void fixed_neighbours(const Stencil<T> &S, int i, int
     }
 }
 
-template <typename T, typename Load, typename Use>
+// Which loops a kernel holds: all (the stencil decides), or that over the entries
+// alone, for stencils without the unrolled one.  The unrolled loops keep six
+// records in flight and cost the FP32 passes 40 to 48 registers; the loop over the
+// entries waits for one record at a time and wants warps instead (512 x 512
+// hexagonal plane, 20 Depondt steps: 12 bonds 555 us with all loops in 40
+// registers, 447 alone in 32; 18 bonds 729 and 587).
+enum class Nbr { ALL, ENTRIES };
+template <Nbr LOOPS = Nbr::ALL, typename T, typename Load, typename Use>
 __device__ __forceinline__ void for_neighbours(const Stencil<T> &S, int i, int b, int c0, int c1, int c2, Load load,
                                                Use use)
 {
-    if (S.fixed == 6) {
+    if (LOOPS == Nbr::ALL && S.fixed == 6) {
         fixed_neighbours<6>(S, i, c0, c1, c2, load, use);
-    } else if (S.fixed == 4) {
+    } else if (LOOPS == Nbr::ALL && S.fixed == 4) {
         fixed_neighbours<4>(S, i, c0, c1, c2, load, use);
     } else {
         const bool inner = interior_site(S, c0, c1, c2);
@@ -419,14 +426,14 @@ template <typename T> __device__ __forceinline__ v3<T> onsite_field(const Stenci
     return S.nb == 1 ? at(0) : at(b);  // one atom: operands at fixed addresses
 }
 
-template <typename T, typename R>
+template <Nbr LOOPS = Nbr::ALL, typename T, typename R>
 __device__ __forceinline__ v3<T> local_field(const Stencil<T> &S, const R *n, int i, v3<T> ni, int &b)
 {
     int c0, c1, c2;
     decode_site(S, i, b, c0, c1, c2);
     v3<T> B = onsite_field(S, b, ni);
-    for_neighbours(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
-                   [&](const NbrEntry<T> &E, v3<T> v) { B = add_bond(E, v, B); });
+    for_neighbours<LOOPS>(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
+                          [&](const NbrEntry<T> &E, v3<T> v) { B = add_bond(E, v, B); });
     return B;
 }
 

@@ -15,6 +15,7 @@
 // Memory per step: read n, write np and q; read np (stencil) and q (and n
 // for Depondt), write n -- 6 (7) records per spin.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -23,11 +24,16 @@
 #define SPGB_LLG_PDL 1
 #endif
 
-// blocks of 256 per SM the FP32 passes' register allocation is held to (512 x
-// 512 hexagonal plane with the dipole field, 20 steps: 6: 1290 us, 5: 1322, 4:
-// 1340; 1024 x 1024 without: 589, 588, 621)
+// blocks of 256 per SM the FP32 passes' register allocation is held to: with all
+// neighbour loops (512 x 512 hexagonal plane with the dipole field, 20 steps: 6:
+// 1290 us, 5: 1322, 4: 1340; 1024 x 1024 without: 589, 588, 621), and with the loop
+// over the entries alone (512 x 512, 12 bonds, 20 Depondt steps: 8: 447 us, 6: 449;
+// RK4 897 and 911)
 #ifndef SPGB_LLG_MINB
 #define SPGB_LLG_MINB 6
+#endif
+#ifndef SPGB_LLG_MINB_ENTRIES
+#define SPGB_LLG_MINB_ENTRIES 8
 #endif
 
 namespace spgb {
@@ -56,17 +62,33 @@ cudaError_t launch_field(const Stencil<T> &S, const rec_t<T> *n, const rec_t<T> 
 }
 
 // ---------------------------------------------------------------- LLG
+// all: blocks per SM of an FP32 kernel with all neighbour loops
+template <typename T, Nbr LOOPS, int all> struct LlgMinB {
+    static constexpr int value = sizeof(T) == 8 ? 1 : (LOOPS == Nbr::ENTRIES ? SPGB_LLG_MINB_ENTRIES : all);
+};
+// The kernel for a stencil, f(LOOPS).  The loop over the entries alone for one atom
+// per cell in FP32; with several atoms, whose entries differ between neighbouring
+// threads, it gains nothing from more warps (two atoms with nine bonds each, 20
+// Depondt steps: 449 us, 427 with all loops), and FP64 is bound by its pipe (12 bonds:
+// 2826 and 2134 us).
+template <typename T, typename F> auto by_loops(const Stencil<T> &S, F &&f)
+{
+    if constexpr (sizeof(T) == 4)
+        if (!S.fixed && S.nb == 1) return f(std::integral_constant<Nbr, Nbr::ENTRIES>{});
+    return f(std::integral_constant<Nbr, Nbr::ALL>{});
+}
+
 // Per-spin bodies of the two passes, shared by the grid kernels (records in
 // global memory) and the single-CTA kernel (records in shared memory).
 // (r: the replica within a batch, whose noise amplitudes and thermal stream
 // the predictor uses; the caller offsets the record pointers.)
-template <typename T, int SOLVER, typename R>
+template <typename T, int SOLVER, Nbr LOOPS = Nbr::ALL, typename R>
 __device__ __forceinline__ void pred_spin(const Stencil<T> &S, const R *n, const rec_t<T> *Bdd, R *np, R *q,
                                           const LlgConst<T> &c, int i, int r = 0)
 {
     int b;
     v3<T> ni = ld(n, i);
-    v3<T> B = local_field(S, n, i, ni, b);
+    v3<T> B = local_field<LOOPS>(S, n, i, ni, b);
     if (Bdd) B = B + ldl2(Bdd, i);
     v3<T> Bth = mk(T(0), T(0), T(0));
     if (c.thermal) Bth = noise_amp(c, r, b) * box_muller(thermal_bits(c, (uint32_t)i, (uint32_t)r), T(0));
@@ -89,13 +111,13 @@ __device__ __forceinline__ void pred_spin(const Stencil<T> &S, const R *n, const
     }
 }
 
-template <typename T, int SOLVER, typename R>
+template <typename T, int SOLVER, Nbr LOOPS = Nbr::ALL, typename R>
 __device__ __forceinline__ void corr_spin(const Stencil<T> &S, R *n, const R *np, const R *q, const rec_t<T> *Bdd,
                                           const LlgConst<T> &c, int i)
 {
     int b;
     v3<T> p = ld(np, i);
-    v3<T> B = local_field(S, np, i, p, b);
+    v3<T> B = local_field<LOOPS>(S, np, i, p, b);
     if (Bdd) B = B + ldl2(Bdd, i);
     v3<T> Ap = llg_A(c.cA[b], c.alpha, p, B);
     v3<T> qi = ld(q, i);
@@ -109,10 +131,10 @@ __device__ __forceinline__ void corr_spin(const Stencil<T> &S, R *n, const R *np
     }
 }
 
-template <typename T, int SOLVER>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_llg_pred(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ n,
-                                                     const rec_t<T> *__restrict__ Bdd, rec_t<T> *__restrict__ np,
-                                                     rec_t<T> *__restrict__ q, const LlgConst<T> c)
+template <typename T, int SOLVER, Nbr LOOPS>
+__global__ void __launch_bounds__(kBlock, (LlgMinB<T, LOOPS, SPGB_LLG_MINB>::value))
+    k_llg_pred(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ n, const rec_t<T> *__restrict__ Bdd,
+               rec_t<T> *__restrict__ np, rec_t<T> *__restrict__ q, const LlgConst<T> c)
 {
     allow_dependents();
     wait_prerequisite(n, Bdd);  // they come from the kernels before
@@ -120,20 +142,20 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_
     if (i >= S.N) return;
     int r = blockIdx.y;  // replica
     size_t o = (size_t)r * S.N;
-    pred_spin<T, SOLVER>(S, n + o, Bdd, np + o, q + o, c, i, r);
+    pred_spin<T, SOLVER, LOOPS>(S, n + o, Bdd, np + o, q + o, c, i, r);
 }
 
-template <typename T, int SOLVER>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_LLG_MINB : 1) k_llg_corr(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n,
-                                                     const rec_t<T> *__restrict__ np, const rec_t<T> *__restrict__ q,
-                                                     const rec_t<T> *__restrict__ Bdd, const LlgConst<T> c)
+template <typename T, int SOLVER, Nbr LOOPS>
+__global__ void __launch_bounds__(kBlock, (LlgMinB<T, LOOPS, SPGB_LLG_MINB>::value))
+    k_llg_corr(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n, const rec_t<T> *__restrict__ np,
+               const rec_t<T> *__restrict__ q, const rec_t<T> *__restrict__ Bdd, const LlgConst<T> c)
 {
     allow_dependents();
     wait_prerequisite(n, np, q, Bdd);  // they come from the kernels before
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S.N) return;
     size_t o = (size_t)blockIdx.y * S.N;  // replica
-    corr_spin<T, SOLVER>(S, n + o, np + o, q + o, Bdd, c, i);
+    corr_spin<T, SOLVER, LOOPS>(S, n + o, np + o, q + o, Bdd, c, i);
 }
 
 // A batch of different lattices: each block belongs to one system, whose
@@ -281,15 +303,14 @@ cudaError_t launch_llg_pred(int solver, const Stencil<T> &S, const rec_t<T> *n, 
                             rec_t<T> *q, const LlgConst<T> &c, cudaStream_t st)
 {
     if (S.N == 0) return cudaSuccess;
-    int bs = llg_block((long)S.N * llg_reps(c));
-    cudaError_t e;
-    if (solver == SP_HEUN)
-        e = launch_llg_kernel(k_llg_pred<T, SP_HEUN>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, Bdd, np, q, c);
-    else if (solver == SP_SIB)
-        e = launch_llg_kernel(k_llg_pred<T, SP_SIB>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, Bdd, np, q, c);
-    else
-        e = launch_llg_kernel(k_llg_pred<T, SP_DEPONDT>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, Bdd, np, q, c);
-    return e;
+    const int bs = llg_block((long)S.N * llg_reps(c));
+    const dim3 g(blocks_for(S.N, bs), llg_reps(c));
+    auto go = [&](auto kern) { return launch_llg_kernel(kern, g, dim3(bs), 0, st, S, n, Bdd, np, q, c); };
+    return by_loops<T>(S, [&](auto l) {
+        if (solver == SP_HEUN) return go(k_llg_pred<T, SP_HEUN, l()>);
+        if (solver == SP_SIB) return go(k_llg_pred<T, SP_SIB, l()>);
+        return go(k_llg_pred<T, SP_DEPONDT, l()>);
+    });
 }
 
 template <typename T>
@@ -297,15 +318,14 @@ cudaError_t launch_llg_corr(int solver, const Stencil<T> &S, rec_t<T> *n, const 
                             const rec_t<T> *Bdd, const LlgConst<T> &c, cudaStream_t st)
 {
     if (S.N == 0) return cudaSuccess;
-    int bs = llg_block((long)S.N * llg_reps(c));
-    cudaError_t e;
-    if (solver == SP_HEUN)
-        e = launch_llg_kernel(k_llg_corr<T, SP_HEUN>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, np, q, Bdd, c);
-    else if (solver == SP_SIB)
-        e = launch_llg_kernel(k_llg_corr<T, SP_SIB>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, np, q, Bdd, c);
-    else
-        e = launch_llg_kernel(k_llg_corr<T, SP_DEPONDT>, dim3(blocks_for(S.N, bs), llg_reps(c)), dim3(bs), 0, st, S, n, np, q, Bdd, c);
-    return e;
+    const int bs = llg_block((long)S.N * llg_reps(c));
+    const dim3 g(blocks_for(S.N, bs), llg_reps(c));
+    auto go = [&](auto kern) { return launch_llg_kernel(kern, g, dim3(bs), 0, st, S, n, np, q, Bdd, c); };
+    return by_loops<T>(S, [&](auto l) {
+        if (solver == SP_HEUN) return go(k_llg_corr<T, SP_HEUN, l()>);
+        if (solver == SP_SIB) return go(k_llg_corr<T, SP_SIB, l()>);
+        return go(k_llg_corr<T, SP_DEPONDT, l()>);
+    });
 }
 
 // ---------------------------------------------------------------- RK4
@@ -313,8 +333,8 @@ cudaError_t launch_llg_corr(int solver, const Stencil<T> &S, rec_t<T> *n, const 
 // the same thermal field in every stage: k = y x A at the stage state y (src),
 // acc accumulates k1 + 2 k2 + 2 k3, the next stage state n + c dt k goes to
 // dst; stage 3 writes normalise(n + dt/6 (acc + k4)) to n.
-template <typename T, int STAGE>
-__global__ void __launch_bounds__(kBlock) k_rk4(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n,
+template <typename T, int STAGE, Nbr LOOPS>
+__global__ void __launch_bounds__(kBlock, (LlgMinB<T, LOOPS, 5>::value)) k_rk4(const __grid_constant__ Stencil<T> S, rec_t<T> *__restrict__ n,
                                                 const rec_t<T> *__restrict__ src, rec_t<T> *__restrict__ dst,
                                                 rec_t<T> *__restrict__ acc, const rec_t<T> *__restrict__ Bdd,
                                                 const LlgConst<T> c)
@@ -331,7 +351,7 @@ __global__ void __launch_bounds__(kBlock) k_rk4(const __grid_constant__ Stencil<
     acc += o;
     int b;
     v3<T> y = ld(src, i);
-    v3<T> B = local_field(S, src, i, y, b);
+    v3<T> B = local_field<LOOPS>(S, src, i, y, b);
     if (Bdd) B = B + ldl2(Bdd, i);
     if (c.thermal) B = B + noise_amp(c, r, b) * box_muller(thermal_bits(c, (uint32_t)i, (uint32_t)r), T(0));
     v3<T> k = cross(y, llg_A(c.cA[b], c.alpha, y, B));
@@ -352,13 +372,16 @@ cudaError_t launch_rk4_stage(int stage, const Stencil<T> &S, rec_t<T> *n, const 
                              rec_t<T> *acc, const rec_t<T> *Bdd, const LlgConst<T> &c, cudaStream_t st)
 {
     if (S.N == 0) return cudaSuccess;
-    dim3 g(blocks_for(S.N), llg_reps(c));
-    switch (stage) {
-    case 0: return launch_llg_kernel(k_rk4<T, 0>, g, dim3(kBlock), 0, st, S, n, src, dst, acc, Bdd, c);
-    case 1: return launch_llg_kernel(k_rk4<T, 1>, g, dim3(kBlock), 0, st, S, n, src, dst, acc, Bdd, c);
-    case 2: return launch_llg_kernel(k_rk4<T, 2>, g, dim3(kBlock), 0, st, S, n, src, dst, acc, Bdd, c);
-    default: return launch_llg_kernel(k_rk4<T, 3>, g, dim3(kBlock), 0, st, S, n, src, dst, acc, Bdd, c);
-    }
+    const dim3 g(blocks_for(S.N), llg_reps(c));
+    auto go = [&](auto kern) { return launch_llg_kernel(kern, g, dim3(kBlock), 0, st, S, n, src, dst, acc, Bdd, c); };
+    return by_loops<T>(S, [&](auto l) {
+        switch (stage) {
+        case 0: return go(k_rk4<T, 0, l()>);
+        case 1: return go(k_rk4<T, 1, l()>);
+        case 2: return go(k_rk4<T, 2, l()>);
+        default: return go(k_rk4<T, 3, l()>);
+        }
+    });
 }
 
 // ---------------------------------------------------------------- energy
