@@ -448,19 +448,19 @@ __device__ __forceinline__ void compensate(float t, float &hi, float &lo)
     hi = s.hi;
     lo += s.lo;
 }
-template <typename R>
+template <Nbr LOOPS = Nbr::ALL, typename R>
 __device__ __forceinline__ v3<float> local_field_comp(const Stencil<float> &S, const R *n, int i, v3<float> ni, int &b,
                                                       v3<float> &lo)
 {
     int c0, c1, c2;
     decode_site(S, i, b, c0, c1, c2);
     v3<float> B = onsite_field(S, b, ni), l = mk(0.f, 0.f, 0.f);
-    for_neighbours(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
-                   [&](const NbrEntry<float> &E, v3<float> v) {
-                       compensate(fmaf(E.J, v.x, fmaf(v.y, E.Dz, -__fmul_rn(v.z, E.Dy))), B.x, l.x);
-                       compensate(fmaf(E.J, v.y, fmaf(v.z, E.Dx, -__fmul_rn(v.x, E.Dz))), B.y, l.y);
-                       compensate(fmaf(E.J, v.z, fmaf(v.x, E.Dy, -__fmul_rn(v.y, E.Dx))), B.z, l.z);
-                   });
+    for_neighbours<LOOPS>(S, i, b, c0, c1, c2, [&](int j) { return ld(n, j); },
+                          [&](const NbrEntry<float> &E, v3<float> v) {
+                              compensate(fmaf(E.J, v.x, fmaf(v.y, E.Dz, -__fmul_rn(v.z, E.Dy))), B.x, l.x);
+                              compensate(fmaf(E.J, v.y, fmaf(v.z, E.Dx, -__fmul_rn(v.x, E.Dz))), B.y, l.y);
+                              compensate(fmaf(E.J, v.z, fmaf(v.x, E.Dy, -__fmul_rn(v.y, E.Dx))), B.z, l.z);
+                          });
     lo = l;
     return B;
 }

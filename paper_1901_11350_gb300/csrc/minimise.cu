@@ -588,7 +588,7 @@ struct NoPost2 {
     __device__ void operator()(int) const {}
 };
 
-template <typename T, typename R>
+template <typename T, Nbr LOOPS = Nbr::ALL, typename R>
 __device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
                                              const Stencil<T> *__restrict__ S, const R *x, R *G, double *part,
                                              unsigned *cnt, double *scal)
@@ -614,7 +614,7 @@ __device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__
         v3<T> B;
         if constexpr (std::is_same<T, float>::value) {
             v3<T> lo;
-            B = local_field_comp(St, xb, i, ni, b, lo);
+            B = local_field_comp<LOOPS>(St, xb, i, ni, b, lo);
             // r[0] collects n.(B + Bz), B = hi + lo; the -1/2 follows at the end
             acc_add(r[0], ni, B);
             acc_add(r[0], ni, mk(St.Bz[b][0], St.Bz[b][1], St.Bz[b][2]));
@@ -652,12 +652,12 @@ __device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__
 }
 static_assert(kE == 0 && kL2 == 1 && kGM == 6 && kVF == 7, "the field pass writes slots 0..7 (7: padding)");
 
-template <typename T>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_GF_MINB : 1) k_g_field(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                                    const Stencil<T> *__restrict__ S, const rec_t<T> *__restrict__ x,
-                                                    rec_t<T> *__restrict__ G, double *part, unsigned *cnt, double *scal)
+template <typename T, Nbr LOOPS>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_GF_MINB : 1)
+    k_g_field(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img, const Stencil<T> *__restrict__ S,
+              const rec_t<T> *__restrict__ x, rec_t<T> *__restrict__ G, double *part, unsigned *cnt, double *scal)
 {
-    g_field_body<T>(blockIdx.x, blk, img, S, x, G, part, cnt, scal);
+    g_field_body<T, LOOPS>(blockIdx.x, blk, img, S, x, G, part, cnt, scal);
 }
 
 // mode 0: F only; 1: v from memory (the call's first iteration); 2: v = c F,
@@ -1104,8 +1104,15 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
     unsigned *cnt = (unsigned *)s->cnt.p;
     double dth_m = a.dt / (2.0 * a.mass), dt2_2m = a.dt * a.dt / (2.0 * a.mass);
     const CoefArgs ca{a.k, a.w, a.climbing, a.w != 0.0};
+    // FP32 batches of chains without the unrolled neighbour loops take the kernel
+    // with the loop over the entries alone, which does not spill (20 images of 128 x
+    // 128 spins, 10 iterations: 18 bonds 734 -> 665 us, 12 bonds 623 -> 570, two atoms
+    // with nine 546 -> 494)
+    bool entries = sizeof(T) == 4;
+    for (const Stencil<T> &sc : stencils) entries = entries && !sc.fixed;
+    const auto field = entries ? k_g_field<T, sizeof(T) == 4 ? Nbr::ENTRIES : Nbr::ALL> : k_g_field<T, Nbr::ALL>;
     auto forces = [&](int mode, cudaStream_t ss) {
-        k_g_field<T><<<n_blk, kBlock, 0, ss>>>(B, I, Sd, x, G, part, cnt, scal);
+        field<<<n_blk, kBlock, 0, ss>>>(B, I, Sd, x, G, part, cnt, scal);
         k_g_coefs<T><<<n_img, 32, 0, ss>>>(I, scal, ca);
         k_g_force<T><<<n_blk, kBlock, 0, ss>>>(B, I, x, v, F, G, dth_m, mode, part, cnt, scal);
     };

@@ -58,3 +58,25 @@ def test_batch_of_lattices_gives_the_bits_of_single_calls(solver):
         c.set_option("generic_stencil", 1)
         y = _step(c, c.spins(n0[off[k]:off[k + 1]]), solver, 5, T=T, replica=k)
         assert (x[off[k]:off[k + 1]] == y).all(), k
+
+
+@pytest.mark.parametrize("name", ["hex_two_shells", "hex_three_shells_open"])
+def test_gneb_gives_the_bits_of_the_persistent_kernel_and_of_a_batch(name):
+    g, h = SYSTEMS[name]
+    M = 6
+    ctxs = [B.Context(g, h, "f32"), B.Context(g, h, "f32"), B.Context(g, dict(h, J=[1.0]), "f32")]
+    ctxs[1].set_option("gneb_persistent", 1)
+    n0 = np.stack([I.perturbed(I.ferromagnet(ctxs[0].N, (0.3 * m, 0.1, 1.0)), 0.2, m) for m in range(M)])
+    out = []
+    for c in ctxs[:2]:
+        x = c.spins(n0)
+        v = x * 0
+        E, F = c.gneb_step(x, v, n_iter=12, dt=0.05)
+        assert c.sync_status()[0] == 0
+        out.append((x, v, E, F))
+    assert all((a == b).all() for a, b in zip(*out))
+    # beside a chain with the unrolled loop
+    x = ctxs[0].spins(np.concatenate([n0.reshape(-1, 3)] * 2))
+    v = x * 0
+    E, F = B.gneb_batch_step([ctxs[0], ctxs[2]], x, v, [0, M * ctxs[0].N], [M, M], n_iter=12, dt=0.05)
+    assert (x[:M * ctxs[0].N].reshape(out[0][0].shape) == out[0][0]).all() and (E[:M] == out[0][2]).all()
