@@ -201,8 +201,6 @@ template <typename T> struct alignas(16) NbrEntry {
     unsigned side;  // bits 0..5: d0 < 0, d0 > 0, d1 < 0, d1 > 0, d2 < 0, d2 > 0
     int jb, d0, d1, d2;
 };
-// most entries of a stencil whose neighbour loop is unrolled (Stencil::fixed)
-constexpr int kFixedNbr = 6;
 
 // Division of a non-negative int below 2^31 by a fixed positive divisor d
 // as q = (umulhi(n, m) + n) >> s with s = ceil(log2 d) and
@@ -251,24 +249,17 @@ template <typename T> struct alignas(16) Stencil {
 
 static_assert(sizeof(Stencil<float>) % 16 == 0 && sizeof(Stencil<double>) % 16 == 0, "16-byte copies of a stencil");
 
-// Copy of the part of a stencil in global memory that is in use (header and
-// the entries of every basis atom) into shared memory, by the whole block;
-// the block's later per-neighbour reads then come from shared memory.  The
-// header and the first entries are copied before their number is looked at:
-// one trip to memory for the common stencils.
+// Copy of the part of a stencil in global memory that is in use (header and the
+// ne entries of all basis atoms) into shared memory, by the whole block (a
+// barrier publishes it); the block's per-neighbour reads then come from there.
+// The number of entries comes with the block's tables: one trip to memory.
 template <typename T>
-__device__ __forceinline__ void stage_stencil(const Stencil<T> *__restrict__ g, Stencil<T> *s)
+__device__ __forceinline__ void copy_stencil(const Stencil<T> *__restrict__ g, Stencil<T> *s, int ne)
 {
-    constexpr int kFirst = (int)((offsetof(Stencil<T>, e) + kFixedNbr * sizeof(NbrEntry<T>) + 15) / 16);
+    const int n16 = (int)((offsetof(Stencil<T>, e) + (size_t)ne * sizeof(NbrEntry<T>) + 15) / 16);
     const uint4 *src = reinterpret_cast<const uint4 *>(g);
     uint4 *dst = reinterpret_cast<uint4 *>(s);
-    for (int k = threadIdx.x; k < kFirst; k += blockDim.x) dst[k] = src[k];
-    __syncthreads();
-    const int ne = s->off[s->nb];
-    if (ne <= kFixedNbr) return;
-    const int n16 = (int)((offsetof(Stencil<T>, e) + (size_t)ne * sizeof(NbrEntry<T>) + 15) / 16);
-    for (int k = kFirst + threadIdx.x; k < n16; k += blockDim.x) dst[k] = src[k];
-    __syncthreads();
+    for (int k = threadIdx.x; k < n16; k += blockDim.x) dst[k] = src[k];
 }
 
 // Periodic wrap for |d| <= n (checked on the host); -1 across an open edge.

@@ -41,7 +41,7 @@ struct ImgInfo {
     int spt;   // spins per thread (GNEB passes; 1 elsewhere)
 };
 struct alignas(16) BlkInfo {
-    int g, t, chain;  // image, block of the image, the image's chain
+    int g, t, chain, ne;  // image, block of the image, the image's chain, its stencil's entries
 };
 
 // per-image scalar slots (kS doubles per image): energy, squared geodesic
@@ -598,7 +598,8 @@ __device__ __forceinline__ void g_field_body(int vb, const BlkInfo *__restrict__
     // the chain's stencil, staged in shared memory for the neighbour loop
     __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
     Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
-    stage_stencil(S + bi.chain, &St);
+    copy_stencil(S + bi.chain, &St, bi.ne);
+    __syncthreads();
     const long long base = im.spin0 + (long long)im.nu * im.N;
     const R *xb = x + base;
     const bool has_p = im.nu < im.M - 1, has_m = im.nu > 0;
@@ -914,7 +915,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_b
     const ImgInfo im = img[bi.g];
     __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
     Stencil<T> &St = *reinterpret_cast<Stencil<T> *>(st_raw);
-    stage_stencil(S + bi.chain, &St);
+    copy_stencil(S + bi.chain, &St, bi.ne);
+    __syncthreads();
     allow_dependents();
     wait_prerequisite(x, v, F, scal, state);  // state, scalars and records come from the kernels before
     if (mode && state[2 * bi.g + 1] == 0) return;
@@ -965,7 +967,7 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
         int N = stencils[c].N;
         int bpi = blocks_for(N > 0 ? N : 1);
         ImgInfo im{spin0[c], N, c, 0, 1, c, (int)blk.size(), bpi, -1, 1};
-        for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{c, t, c});
+        for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{c, t, c, stencils[c].off[stencils[c].nb]});
         img.push_back(im);
         total = std::max(total, spin0[c] + (long long)N);
     }
@@ -1019,7 +1021,7 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
         for (int c = 0; c < C; ++c)
             if (hs[2 * c + 1]) {
                 img[c].blk0 = (int)act.size();
-                for (int t = 0; t < img[c].bpi; ++t) act.push_back(BlkInfo{c, t, c});
+                for (int t = 0; t < img[c].bpi; ++t) act.push_back(BlkInfo{c, t, c, stencils[c].off[stencils[c].nb]});
             }
         if (act.empty()) break;
         if (4 * (long long)act.size() <= 3LL * n_act) {
@@ -1067,7 +1069,7 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
         for (int nu = 0; nu < M[c]; ++nu) {
             int kind = a.kinds ? a.kinds[g0 + nu] : -1;
             ImgInfo im{spin0[c], N, c, nu, M[c], g0, (int)blk.size(), bpi, kind, spt};
-            for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{(int)img.size(), t, c});
+            for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{(int)img.size(), t, c, stencils[c].off[stencils[c].nb]});
             img.push_back(im);
         }
         total = std::max(total, spin0[c] + (long long)M[c] * N);
