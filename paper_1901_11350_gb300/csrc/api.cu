@@ -596,7 +596,6 @@ int llg_batch_run(sp_ctx *const *ctxs, int n_sys, void *spins, const long long *
         LlgSys<T> s{};
         s.spin0 = spin0[k];
         s.N = c->N;
-        s.ne = sten[k].off[sten[k].nb];
         s.replica = p->replica + (uint32_t)k;
         for (int b = 0; b < c->nb; ++b) {  // as llg_const does for one lattice
             double mu = c->mu_s[b] * kMuB;

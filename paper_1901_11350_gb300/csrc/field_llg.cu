@@ -160,17 +160,13 @@ __global__ void __launch_bounds__(kBlock, (LlgMinB<T, LOOPS, SPGB_LLG_MINB>::val
 
 // A batch of different lattices: each block belongs to one system, whose
 // constants (prefactors, noise amplitudes, thermal stream) the block takes
-// into a shared-memory copy of the common constants, and its stencil beside
-// them (read from global memory by every neighbour loop, eight lattices half of
-// which have 12 bonds took 519 us for 32 Heun steps, 502 with the copy); then the
-// per-spin bodies of the single-lattice kernels run unchanged, so every system
-// gets the result a call on it alone gives.
+// into a shared-memory copy of the common constants; then the per-spin
+// bodies of the single-lattice kernels run unchanged, so every system gets
+// the result a call on it alone gives.
 template <typename T>
-__device__ __forceinline__ const LlgConst<T> &batch_const(const LlgConst<T> &c, const LlgSys<T> &s,
-                                                          const Stencil<T> *g, Stencil<T> *S)
+__device__ __forceinline__ const LlgConst<T> &batch_const(const LlgConst<T> &c, const LlgSys<T> &s)
 {
     __shared__ LlgConst<T> cs;
-    copy_stencil(g, S, s.ne);
     if (threadIdx.x == 0) {
         cs = c;
         for (int b = 0; b < SP_MAX_BASIS; ++b) {
@@ -191,13 +187,11 @@ __global__ void __launch_bounds__(kBlock) k_llg_bpred(const int2 *__restrict__ b
                                                       rec_t<T> *__restrict__ np, rec_t<T> *__restrict__ q,
                                                       const LlgConst<T> c)
 {
-    // the tables do not change while kernels are in flight
-    const int2 bt = blk[blockIdx.x];
-    __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
-    Stencil<T> &S = *reinterpret_cast<Stencil<T> *>(st_raw);
-    const LlgConst<T> &cs = batch_const(c, sys[bt.x], Sv + bt.x, &S);
     allow_dependents();
     wait_prerequisite(n);  // it comes from the kernels before
+    const int2 bt = blk[blockIdx.x];
+    const LlgConst<T> &cs = batch_const(c, sys[bt.x]);
+    const Stencil<T> &S = Sv[bt.x];
     int i = bt.y * kBlock + threadIdx.x;
     if (i >= S.N) return;
     size_t o = (size_t)sys[bt.x].spin0;
@@ -210,13 +204,11 @@ __global__ void __launch_bounds__(kBlock) k_llg_bcorr(const int2 *__restrict__ b
                                                       const rec_t<T> *__restrict__ np, const rec_t<T> *__restrict__ q,
                                                       const LlgConst<T> c)
 {
-    // the tables do not change while kernels are in flight
-    const int2 bt = blk[blockIdx.x];
-    __shared__ __align__(16) unsigned char st_raw[sizeof(Stencil<T>)];
-    Stencil<T> &S = *reinterpret_cast<Stencil<T> *>(st_raw);
-    const LlgConst<T> &cs = batch_const(c, sys[bt.x], Sv + bt.x, &S);
     allow_dependents();
     wait_prerequisite(n, np, q);  // they come from the kernels before
+    const int2 bt = blk[blockIdx.x];
+    const LlgConst<T> &cs = batch_const(c, sys[bt.x]);
+    const Stencil<T> &S = Sv[bt.x];
     int i = bt.y * kBlock + threadIdx.x;
     if (i >= S.N) return;
     size_t o = (size_t)sys[bt.x].spin0;

@@ -67,8 +67,8 @@ template <typename T> __device__ __forceinline__ uint4 thermal_bits(const LlgCon
 // single call).
 template <typename T> struct LlgSys {
     long long spin0;
-    int N, ne;  // spins, entries of the stencil
-    uint32_t replica, unused;
+    int N;
+    uint32_t replica;
     T cA[SP_MAX_BASIS], sig[SP_MAX_BASIS];
 };
 
