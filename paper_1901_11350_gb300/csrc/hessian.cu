@@ -308,15 +308,17 @@ __global__ void __launch_bounds__(kLzB) k_lz_begin(const __grid_constant__ Stenc
     if (threadIdx.x == 0) partN[blockIdx.x] = r;
 }
 
-// H w for a tangent w, not scaled: -P (sum_j J w_j + w_j x D + 2 K (Kh.w) Kh) + (n.B) w
+// H u for u = scale w, w tangent: -P (sum_j J u_j + u_j x D + 2 K (Kh.u) Kh) + (n.B) u; u: that of spin i
 template <typename T>
-__device__ __forceinline__ v3<T> lz_product(const Stencil<T> &S, const rec_t<T> *w, int i, v3<T> ni, v3<T> u, T nB)
+__device__ __forceinline__ v3<T> lz_product(const Stencil<T> &S, const rec_t<T> *w, int i, v3<T> ni, v3<T> u, T nB,
+                                            T scale)
 {
     int bs, c0, c1, c2;
     decode_site(S, i, bs, c0, c1, c2);
     const v3<T> kh = mk(S.Kh[bs][0], S.Kh[bs][1], S.Kh[bs][2]);
     v3<T> L = (T(2) * S.K[bs] * dot(kh, u)) * kh;
-    for_neighbours(S, i, bs, c0, c1, c2, [&](int j) { return ldg2(w, j); },  // tangent already: no projection here
+    auto load = [&](int j) { return sizeof(T) == 4 ? scale * ldg2(w, j) : ldg2(w, j); };  // tangent: no projection here
+    for_neighbours(S, i, bs, c0, c1, c2, load,
                    [&](const NbrEntry<T> &E, v3<T> v) {
                        L.x = fma(-v.z, E.Dy, fma(v.y, E.Dz, fma(E.J, v.x, L.x)));
                        L.y = fma(-v.x, E.Dz, fma(v.z, E.Dx, fma(E.J, v.y, L.y)));
@@ -357,28 +359,45 @@ __global__ void __launch_bounds__(kLzB) k_lz_apply(const __grid_constant__ Stenc
             }
         }
     }
-    // the product is linear: it is formed from the unscaled w while the norm
-    // is being summed
     rec_t<T> *q = Q + (size_t)k * S.N;
-    int i = blockIdx.x * kLzB + threadIdx.x;
-    v3<T> u = mk(T(0), T(0), T(0)), h = u;
-    if (i < S.N) {
-        u = ldg2(w, i);
-        h = lz_product(S, w, i, ldc(n, i), u, nB[i]);
-    }
-    __syncthreads();
-    const T inv = (T)s_inv;
-    if (inv == T(0)) return;
     typename LzAcc<T>::type s{};
-    while (i < S.N) {
-        const v3<T> qi = inv * u, r = inv * h;
-        st(q, i, qi);
-        st(wn, i, r);
-        s = s + lz_dot(qi, r);
-        i += gridDim.x * kLzB;
-        if (i >= S.N) break;
-        u = ldg2(w, i);
-        h = lz_product(S, w, i, ldc(n, i), u, nB[i]);
+    int i = blockIdx.x * kLzB + threadIdx.x;
+    if constexpr (sizeof(T) == 4) {
+        // FP32: the product of the vector as it is stored.  That of the unscaled w
+        // (below) is not its product to the last bits, and shows in the mode:
+        // 8.5e-7 off (geometric mean of 150 states, 50 x 50, 40 vectors), 7.6e-7
+        // with the product of q; 1.02e-6 and 0.91e-6 at 64 x 64 and 64 vectors (128 x
+        // 128, 64 vectors: 1.59 ms, and 1.67 for the norm that comes first)
+        __syncthreads();
+        const T inv = (T)s_inv;
+        if (inv == T(0)) return;
+        for (; i < S.N; i += gridDim.x * kLzB) {
+            const v3<T> qi = inv * ldg2(w, i), r = lz_product(S, w, i, ldc(n, i), qi, nB[i], inv);
+            st(q, i, qi);
+            st(wn, i, r);
+            s = s + lz_dot(qi, r);
+        }
+    } else {
+        // FP64: the product is linear, and is formed from the unscaled w while the
+        // norm is being summed
+        v3<T> u = mk(T(0), T(0), T(0)), h = u;
+        if (i < S.N) {
+            u = ldg2(w, i);
+            h = lz_product(S, w, i, ldc(n, i), u, nB[i], T(1));
+        }
+        __syncthreads();
+        const T inv = (T)s_inv;
+        if (inv == T(0)) return;
+        while (i < S.N) {
+            const v3<T> qi = inv * u, r = inv * h;
+            st(q, i, qi);
+            st(wn, i, r);
+            s = s + lz_dot(qi, r);
+            i += gridDim.x * kLzB;
+            if (i >= S.N) break;
+            u = ldg2(w, i);
+            h = lz_product(S, w, i, ldc(n, i), u, nB[i], T(1));
+        }
     }
     allow_dependents();
     const double r = block_sum(s);
