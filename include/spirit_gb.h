@@ -250,16 +250,20 @@ int sp_llg_step(sp_ctx *ctx, void *n_dev, const sp_llg_params *p, int n_steps, v
  * temperature T[r] (K, host array) and the thermal stream p->replica + r
  * (Philox counter word 3 = 8 (p->replica + r)); p->T is ignored.  Each
  * replica's result is the one sp_llg_step gives that replica alone with
- * p->T = T[r] and p->replica + r, bit for bit: the noise amplitudes are
+ * p->T = T[r] and p->replica + r, bit for bit where both calls take the same
+ * kernels (else within the precision's rounding): the noise amplitudes are
  * computed on the host in FP64 in the same way.  All replicas share one launch per
  * pass (the 27-point path spreads all replicas' (tile, plane) units over the
  * device; batches of two or more do not take the small-lattice single-CTA
- * path, a batch of one is sp_llg_step at T[0]).  Where the 27-point split
- * would give fewer than 8 planes per CTA (unless SP_OPT_PLANES_PER_CTA is
- * set) the per-spin kernels run instead.  Runs of up to 32 steps are
- * replayed from a CUDA graph captured on first use for the launch
- * configuration (up to 4 kept per context; not while `stream` is being
- * captured); their Philox step is read from a device counter the call sets.
+ * path, a batch of one is sp_llg_step at T[0]).  Where the general 27-point
+ * passes' split would give fewer than 8 planes per CTA (unless
+ * SP_OPT_PLANES_PER_CTA is set), and the lean Heun passes are not expected to
+ * be faster, the per-spin kernels run instead; sp_llg_step takes the 27-point
+ * path (a lattice of at most 2048 spins: the small-lattice path) there.  Runs
+ * of up to 32 steps are replayed from a CUDA graph captured on first use for
+ * the launch configuration (up to 4 kept per context; not while `stream` is
+ * being captured); their Philox step is read from a device counter the call
+ * sets.
  * The kernel profiler does not bracket these launches.  Scratch: 2 (RK4:
  * 3) records per spin and replica; the amplitudes are re-uploaded (with a
  * synchronisation of `stream`) only when n_rep, T, dt or alpha change.

@@ -503,18 +503,22 @@ int replicas_run(sp_ctx *c, void *n, const sp_llg_params *p, int n_steps, cudaSt
     for (int r = 0; r < n_rep; ++r) hot = hot || temps[r] > 0;
     k.thermal = (hot && p->alpha > 0) ? 1 : 0;
     bool cub = c->cubic && c->use_cubic;  // all four solvers (a batch has no dipole term)
-    const bool lean = cub && p->solver == SP_HEUN && cubic_lean_taken(c);
-    int per0 = cub ? cubic_per_batch(c, 0, n_rep, lean) : 0, per1 = cub ? cubic_per_batch(c, 1, n_rep, lean) : 0;
-    // runs of a few planes per CTA are mostly the ring's prologue: the
-    // per-spin kernels are faster there (unless the user fixed the split).
-    // The lean passes: 32 steps take about 240 + 0.148 U us for U (32 x 8 tile,
-    // plane) units, the per-spin kernels 140 + 1.04 K us for K thousand spins
-    // (29 replicas of 30^3: 723 and 950 us; 12: 439 and 480; 7: 332 and 320; 29
-    // of 24^3: 514 and 562, of 22^3: 617 and 467, of 16^3: 343 and 260)
-    if (cub && c->zc == 0) {
+    // Runs of a few planes per CTA are mostly the ring's prologue: where the
+    // general passes' split gives fewer than kCubicMinRun the per-spin kernels are
+    // faster (unless the user fixed the split).  Batches that Heun's lean passes are
+    // faster for stay all the same: 32 steps take them about 240 + 0.148 U us for U
+    // (32 x 8 tile, plane) units, and the per-spin kernels 140 + 1.04 K us for K
+    // thousand spins (29 replicas of 30^3: 723 and 950 us; 12: 439 and 480; 7: 332
+    // and 320; 29 of 24^3: 514 and 562, of 22^3: 617 and 467, of 16^3: 343 and 260).
+    // The times alone do not decide: a single call takes the 27-point path, and a
+    // batch that leaves it gives up that call's bits (256 of 16^3 stay, at 1496 us
+    // instead of 1242).
+    bool lean = cub && p->solver == SP_HEUN && cubic_lean_taken(c);
+    if (cub && c->zc == 0 && cubic_per_batch(c, 0, n_rep, false) < kCubicMinRun) {
         const double units = (double)cubic_units(c->nc[0], c->nc[1], c->nc[2]) * n_rep, kspins = 1e-3 * (double)NR;
-        if (lean ? 1.04 * kspins < 100.0 + 0.148 * units : per0 < kCubicMinRun) cub = false;
+        if (!lean || 1.04 * kspins < 100.0 + 0.148 * units) cub = lean = false;
     }
+    const int per0 = cub ? cubic_per_batch(c, 0, n_rep, lean) : 0, per1 = cub ? cubic_per_batch(c, 1, n_rep, lean) : 0;
     auto one_step = [&](const LlgConst<T> &kk, cudaStream_t s) -> cudaError_t {
         if (rk4) {
             const rec_t<T> *src[4] = {nn, np, q, np};
