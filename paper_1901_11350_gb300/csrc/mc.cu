@@ -46,6 +46,13 @@ namespace {
 constexpr int kMcBlock = 256;
 constexpr int kMcGraphSweeps = 16;
 constexpr int kMcMaxRows = 65535;  // blocks along y of a grid, at most
+// From this many blocks on (two per SM) a colour whose spins leave a twentieth of
+// the blocks' threads idle packs the replicas' trials instead of giving every
+// replica its own blocks.  32 sweeps, packed and not: 200 replicas of 17^3 (289
+// spins a colour) 2387 and 2593 us, of 15^3 (1125) 636 and 691, 1500 of 17^3 8290
+// and 9467, of 18^3 (2916) 4589 and 4833; 29 of 13^3 (58 blocks) 1346 and 1054, 200
+// of 16^3 (none idle) 643 and 628.
+constexpr long long kMcPackBlocks = 304;
 
 struct McColour {
     int k, res;            // sum colouring: (c0 + c1 + c2) mod k == res; k = 0: the product colouring
@@ -57,6 +64,7 @@ struct McColour {
     int s0, s1, s2;        // cells of this colour per direction
     int b;                 // basis atom
     long long per;         // spins of this colour per replica
+    FastDiv fper;          // division by per (per * replicas < 2^31)
 };
 
 // threads of the resident kernel's CTA (FP64: fewer, for the registers)
@@ -219,7 +227,11 @@ __device__ __forceinline__ bool mc_trial(const Stencil<T> &S, const McFaces<T> &
     return ok;
 }
 
-template <typename T, bool DMI, bool FACES>
+// One colour of every replica.  PACK false: a block's trials belong to one
+// replica (row blockIdx.y + k gridDim.y), so its cone and temperature are read
+// once and its accepted trials are counted by the barrier.  PACK true: the
+// replicas' trials follow one another and a block takes 256 of them.
+template <typename T, bool DMI, bool FACES, bool PACK>
 __global__ void __launch_bounds__(kMcBlock) k_mc_colour(const __grid_constant__ Stencil<T> S,
                                                         const __grid_constant__ McFaces<T> F, rec_t<T> *__restrict__ x,
                                                         int n_rep, McColour col, const T *__restrict__ temps,
@@ -229,23 +241,37 @@ __global__ void __launch_bounds__(kMcBlock) k_mc_colour(const __grid_constant__ 
                                                         unsigned long long *__restrict__ acc)
 {
     // replicas x spins of a colour stay below 2^31 (checked on the host):
-    // 32-bit indices, multiply-high divisions.  A block's trials belong to
-    // one replica (row blockIdx.y + k gridDim.y), so its cone and temperature
-    // are read once and its accepted trials are counted by the barrier
-    // (29 replicas of 30^3: 7.3 -> 7.1 us a launch)
-    const int q = (int)blockIdx.x * kMcBlock + (int)threadIdx.x;
-    for (int rep = blockIdx.y; rep < n_rep; rep += gridDim.y) {
-        bool ok = false;
-        if (q < (int)col.per) {
-            int b, c0, c1, c2;
-            int i = mc_site(S, col, q, b, c0, c1, c2);
-            // per replica: the cone as its cosine (once per sweep, from FP64) and
-            // the temperature factor (once per call): no FP64 work per trial
-            ok = mc_trial<DMI, FACES>(S, F, x + (long long)rep * S.N, i, b, c0, c1, c2, rep, *sweep_dev, keys, cosc[rep],
-                                      temps[rep]);
+    // 32-bit indices, multiply-high divisions
+    auto trial = [&](int rep, int q) {
+        int b, c0, c1, c2;
+        int i = mc_site(S, col, q, b, c0, c1, c2);
+        // per replica: the cone as its cosine (once per sweep, from FP64) and
+        // the temperature factor (once per call): no FP64 work per trial
+        return mc_trial<DMI, FACES>(S, F, x + (long long)rep * S.N, i, b, c0, c1, c2, rep, *sweep_dev, keys, cosc[rep],
+                                    temps[rep]);
+    };
+    if constexpr (PACK) {
+        __shared__ unsigned cnt[kMcBlock];
+        cnt[threadIdx.x] = 0;
+        __syncthreads();
+        const int t0 = (int)blockIdx.x * kMcBlock;  // < total: the grid covers total exactly
+        const unsigned t = (unsigned)t0 + threadIdx.x;
+        const int rep0 = fdiv(t0, col.fper);
+        if (t < (unsigned)col.per * (unsigned)n_rep) {
+            const int rep = fdiv((int)t, col.fper);
+            if (trial(rep, (int)t - rep * (int)col.per)) atomicAdd(&cnt[rep - rep0], 1u);
         }
-        const unsigned c = (unsigned)__syncthreads_count(ok);
-        if (threadIdx.x == 0 && c) atomicAdd(&acc[rep], (unsigned long long)c);
+        __syncthreads();
+        // (rep - rep0 < 256: a replica has at least one trial)
+        const unsigned c = cnt[threadIdx.x];
+        if (c) atomicAdd(&acc[rep0 + threadIdx.x], (unsigned long long)c);
+    } else {
+        const int q = (int)blockIdx.x * kMcBlock + (int)threadIdx.x;
+        for (int rep = blockIdx.y; rep < n_rep; rep += gridDim.y) {
+            const bool ok = q < (int)col.per && trial(rep, q);
+            const unsigned c = (unsigned)__syncthreads_count(ok);
+            if (threadIdx.x == 0 && c) atomicAdd(&acc[rep], (unsigned long long)c);
+        }
     }
 }
 
@@ -595,6 +621,7 @@ std::vector<McColour> mc_colours(const Stencil<T> &S)
             c.fkk = make_fastdiv(k);
             c.s0 = c.s1 = c.s2 = 1;
             c.per = (long long)S.N / k;
+            c.fper = make_fastdiv((int)c.per);
             out.push_back(c);
         }
         return out;
@@ -618,7 +645,8 @@ std::vector<McColour> mc_colours(const Stencil<T> &S)
                     c.s2 = (n[2] - r2 + m[2] - 1) / m[2];
                     c.b = b;
                     c.per = (long long)c.s0 * c.s1 * c.s2;
-                            out.push_back(c);
+                    if (c.per) c.fper = make_fastdiv((int)c.per);
+                    out.push_back(c);
                 }
     return out;
 }
@@ -759,8 +787,16 @@ int mc_run(sp_ctx *c, const Stencil<T> &S, void *spins, int n_rep, const double 
     auto sweep = [&](cudaStream_t ss) {
         for (const McColour &col : cols) {
             if (!col.per) continue;
-            const dim3 grid((unsigned)((col.per + kMcBlock - 1) / kMcBlock), (unsigned)std::min(n_rep, kMcMaxRows));
-            k_mc_colour<T, DMI, FACES><<<grid, kMcBlock, 0, ss>>>(S, F, x, n_rep, col, temps, cosc, sw, keys, acc);
+            const long long rows = (col.per + kMcBlock - 1) / kMcBlock;
+            if (rows * n_rep > kMcPackBlocks && 19 * rows * kMcBlock > 20 * col.per) {
+                const long long blocks = (col.per * n_rep + kMcBlock - 1) / kMcBlock;
+                k_mc_colour<T, DMI, FACES, true><<<(unsigned)blocks, kMcBlock, 0, ss>>>(S, F, x, n_rep, col, temps, cosc,
+                                                                                       sw, keys, acc);
+            } else {
+                const dim3 grid((unsigned)rows, (unsigned)std::min(n_rep, kMcMaxRows));
+                k_mc_colour<T, DMI, FACES, false><<<grid, kMcBlock, 0, ss>>>(S, F, x, n_rep, col, temps, cosc, sw, keys,
+                                                                            acc);
+            }
         }
         const McCone<T> cc{acc, cone, cosc, p->target_accept, sw};
         if (p->sample)
