@@ -53,7 +53,7 @@ SOLVER_BYTES = {"heun": {"llg_predictor": 48, "llg_corrector": 48},
 # place of recomputing the stencil on n and the noise.)  RK4 has no two-stage
 # figure and is charged with the design's bytes.
 METHOD_STEP_BYTES = {"heun": 80, "depondt": 80, "sib": 80}
-# the lean FP32 Heun passes (whole 32 x 8 tiles) pack q into the predicted
+# the lean FP32 Heun passes pack q into the predicted
 # record's pad word plus 8 bytes: read n, write n^p|q_x and q_yz (40 B); read
 # those, write n (40 B)
 LEAN_HEUN_BYTES = {"llg_predictor": 40, "llg_corrector": 40}
@@ -274,7 +274,7 @@ def run_gpu(args):
     n = host0.to("cuda")
     kw = dict(solver=args.solver, dt=r["dt"], alpha=r["alpha"],
               T=r["T"] if args.temperature is None else args.temperature, seed=r["seed"], replica=rank)
-    lean = args.solver == "heun" and bool(ctx.get_option("cubic_lean"))
+    lean = args.solver == "heun" and bool(ctx.get_option("heun_lean"))
     bps = LEAN_HEUN_BYTES if lean else SOLVER_BYTES[args.solver]
     bytes_per_step = bps["llg_predictor"] + CORRECTOR_LAUNCHES[args.solver] * bps["llg_corrector"]
     if not args.zc and not args.generic and not args.cubic_rows:

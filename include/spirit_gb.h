@@ -592,7 +592,9 @@ enum {
     /* work of one CTA of the 27-point path, in (32 x 8 column tile, plane)
      * units taken in tile-major order (>= 1); 0 (default): the units spread
      * evenly over one wave of the CTAs the device keeps resident (reading
-     * the option then returns that value once it has been computed) */
+     * the option then returns that value once it has been computed: that of a
+     * Heun call, in units of the tile height SP_OPT_CUBIC_ROWS reads, or where
+     * none has been made that of the other solvers) */
     SP_OPT_PLANES_PER_CTA = 2,
     /* read only: 1 when the 27-point path applies to this Hamiltonian */
     SP_OPT_HAS_CUBIC_PATH = 3,
@@ -646,7 +648,8 @@ enum {
      * spin, bit-identical results) -- FP32 single lattices without the
      * dipole term only, other calls take 1.  Sets both passes; units of
      * SP_OPT_PLANES_PER_CTA are then (32 x 16 tile, plane).  sp_autotune
-     * chooses it per pass.  Reading returns the predictor's value in use */
+     * chooses it per pass.  Reading returns the value the predictor of a Heun
+     * call uses, the lean passes' default of two included */
     SP_OPT_CUBIC_ROWS = 11,
     /* the same for the corrector pass alone */
     SP_OPT_CUBIC_ROWS_CORR = 12,
@@ -657,11 +660,16 @@ enum {
      * give the same bits).  Where neither SP_OPT_CUBIC_ROWS nor a split is set a
      * single lattice takes two columns per thread in the predictor, and in the
      * corrector where they make whole tiles.
-     * 0: always the general passes.  Reading returns 1 when the lean passes
-     * would be taken for a Heun call of this context and its xy plane is cut
-     * into whole column tiles of the tile height in SP_OPT_CUBIC_ROWS (nx a
-     * multiple of 32; ny of 8 with one column per thread, of 16 with two) */
-    SP_OPT_CUBIC_LEAN = 13
+     * 0: always the general passes.  Reading returns 1 when a Heun call of this
+     * context takes the lean passes and its xy plane is cut into whole column
+     * tiles of the height set with SP_OPT_CUBIC_ROWS (nx a multiple of 32; ny
+     * of 8 with one column per thread, of 16 with two); SP_OPT_HEUN_LEAN tells
+     * whether the passes are taken at all */
+    SP_OPT_CUBIC_LEAN = 13,
+    /* read only: 1 when a Heun call of this context takes the lean passes,
+     * whatever its extents (a batch of replicas: where it takes the 27-point
+     * path) */
+    SP_OPT_HEUN_LEAN = 14
 };
 int sp_set_option(sp_ctx *ctx, int option, int value);
 /* Choose the tile height (SP_OPT_CUBIC_ROWS) and the work per CTA of the

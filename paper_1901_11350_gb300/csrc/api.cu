@@ -1512,7 +1512,7 @@ int sp_get_option(const sp_ctx *c, int option, int *value)
         *value = c->use_cubic ? 0 : 1;
         return SP_OK;
     case SP_OPT_PLANES_PER_CTA:
-        *value = c->zc > 0 ? c->zc : c->zc_auto;
+        *value = c->zc > 0 ? c->zc : (c->zc_auto > 0 ? c->zc_auto : c->zc_gen[0]);
         return SP_OK;
     case SP_OPT_HAS_CUBIC_PATH:
         *value = c->cubic ? 1 : 0;
@@ -1524,7 +1524,9 @@ int sp_get_option(const sp_ctx *c, int option, int *value)
         *value = c->use_small ? 1 : 0;
         return SP_OK;
     case SP_OPT_PLANES_PER_CTA_CORR:
-        *value = c->zc_corr > 0 ? c->zc_corr : (c->zc > 0 ? c->zc : c->zc_auto_corr);
+        *value = c->zc_corr > 0 ? c->zc_corr
+                 : c->zc > 0    ? c->zc
+                                : (c->zc_auto_corr > 0 ? c->zc_auto_corr : c->zc_gen[1]);
         return SP_OK;
     case SP_OPT_MC_RESIDENT:
         *value = c->use_mc_resident ? 1 : 0;
@@ -1533,13 +1535,16 @@ int sp_get_option(const sp_ctx *c, int option, int *value)
         *value = c->gneb_persistent;
         return SP_OK;
     case SP_OPT_CUBIC_ROWS:
-        *value = cubic_rows(c, 0);
+        *value = cubic_rows(c, 0, cubic_lean_taken(c));
         return SP_OK;
     case SP_OPT_CUBIC_ROWS_CORR:
-        *value = cubic_rows(c, 1);
+        *value = cubic_rows(c, 1, cubic_lean_taken(c));
         return SP_OK;
     case SP_OPT_CUBIC_LEAN:
         *value = cubic_lean_taken(c) && cubic_lean_fits(c->nc[0], c->nc[1], cubic_rows(c, 0)) ? 1 : 0;  // whole tiles
+        return SP_OK;
+    case SP_OPT_HEUN_LEAN:
+        *value = cubic_lean_taken(c) ? 1 : 0;
         return SP_OK;
     case SP_OPT_WAIT_LIMIT:
         *value = c->wait_limit;
