@@ -657,8 +657,8 @@ enum {
      * passes (without the dipole term; one lattice or a batch of replicas); the
      * same method and stencil, fewer instructions per spin, results equal to the
      * general passes within FP32 rounding (not bit for bit; one and two columns
-     * give the same bits).  Where neither SP_OPT_CUBIC_ROWS nor a split is set a
-     * single lattice takes two columns per thread in the predictor, and in the
+     * give the same bits).  A pass of a single lattice whose columns and split
+     * are not set takes two columns per thread: the predictor always, the
      * corrector where they make whole tiles.
      * 0: always the general passes.  Reading returns 1 when a Heun call of this
      * context takes the lean passes and its xy plane is cut into whole column

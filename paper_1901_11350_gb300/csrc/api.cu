@@ -1468,9 +1468,12 @@ int sp_set_option(sp_ctx *c, int option, int value)
     case SP_OPT_CUBIC_ROWS:
     case SP_OPT_CUBIC_ROWS_CORR:
         if (value != 1 && value != 2) return fail(c, SP_ERR_ARG, "columns per thread: 1 or 2");
-        if (option == SP_OPT_CUBIC_ROWS) c->rows[0] = value;
+        if (option == SP_OPT_CUBIC_ROWS) {
+            c->rows[0] = value;
+            c->rows_set[0] = true;
+        }
         c->rows[1] = value;
-        c->rows_set[option == SP_OPT_CUBIC_ROWS ? 0 : 1] = true;
+        c->rows_set[1] = true;
         c->zc_auto = c->zc_auto_corr = c->zc_gen[0] = c->zc_gen[1] = 0;
         return SP_OK;
     case SP_OPT_CUBIC_LEAN:

@@ -192,14 +192,15 @@ inline bool cubic_lean_taken(const sp_ctx *c)
 {
     return c->lean && c->prec == SP_F32 && c->cubic && c->use_cubic && c->h.dipole == SP_DIPOLE_NONE;
 }
-// Columns per thread of a lean pass: the user's choice, else two in the
+// Columns per thread of a lean pass: the user's choice (of the columns, or of
+// the pass's split, which counts tiles of that height), else two in the
 // predictor (which shares the rows both read and has two independent chains:
 // 1 to 7% faster on ten lattices from 24^3 to 128^3) and two in the corrector
 // where they make whole tiles (5% faster at 128^3, 13% at 64^3; on ragged
 // lattices 2 to 14% slower).
 inline int lean_rows(const sp_ctx *c, int pass)
 {
-    if (c->rows_set[0] || c->rows_set[1] || c->zc > 0 || c->zc_corr > 0) return c->rows[pass];
+    if (c->rows_set[pass] || c->zc > 0 || (pass == 1 && c->zc_corr > 0)) return c->rows[pass];
     return pass == 0 || cubic_lean_fits(c->nc[0], c->nc[1], 2) ? 2 : 1;
 }
 inline int cubic_rows(const sp_ctx *c, int pass, bool lean) { return lean ? lean_rows(c, pass) : cubic_rows(c, pass); }

@@ -40,3 +40,12 @@ def test_split_reads_that_of_the_calls_made():
         c.llg_step(n, 1, solver=solver)
         assert c.get_option("planes_per_cta") >= 1 and c.get_option("planes_per_cta_corr") >= 1
     torch.cuda.synchronize()
+
+
+def test_a_choice_for_the_corrector_leaves_the_predictor_alone():
+    assert _read(_ctx((33, 16, 4), cubic_rows_corr=2)) == (1, 2, 2)
+    assert _read(_ctx((32, 16, 4), cubic_rows_corr=1)) == (1, 2, 1)
+    assert _read(_ctx((32, 16, 4), planes_per_cta_corr=3)) == (1, 2, 1)
+    assert _read(_ctx((32, 16, 4), planes_per_cta=3)) == (1, 1, 1)
+    assert _read(_ctx((32, 16, 4), cubic_rows=1, cubic_rows_corr=2)) == (1, 1, 2)
+    assert _read(_ctx((32, 16, 4), cubic_rows_corr=1, cubic_rows=2)) == (1, 2, 2)
