@@ -407,12 +407,16 @@ __global__ void __launch_bounds__(kMcBlock) k_mc_sample(const __grid_constant__ 
     double s = sh[l % 8][l / 8];
     for (int o = 4; o > 0; o >>= 1) s += mc_xor(s, o);
     if (l % 8 == 0) part[4 * (size_t)blockIdx.x + l / 8] = s;
-    __threadfence();
+    // lane 0 fences for the warp, between its barriers and the ticket
     __syncwarp();
     int last = 0;
-    if (l == 0) last = atomicAdd(&tickets[rep], 1u) == (unsigned)(bpr - 1);
+    if (l == 0) {
+        __threadfence();
+        last = atomicAdd(&tickets[rep], 1u) == (unsigned)(bpr - 1);
+        __threadfence();
+    }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
-    __threadfence();
+    __syncwarp();
     // the replica's last block: lane 8 k + j sums value k of partials j,
     // j + 8, ..., then the lanes combine (a fixed order); every lane has all
     // four totals and lanes 0..5 add to a statistic each

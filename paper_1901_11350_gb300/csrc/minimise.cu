@@ -249,12 +249,17 @@ __device__ __forceinline__ void image_sums(V (&v)[NS], V m, double *__restrict__
     }
     if (l % LPV == 0) part[(size_t)blk * ROW + l / LPV] = a;
     if (MAX && l == 0) part[(size_t)blk * ROW + NS] = mx;
-    __threadfence();
+    // the fences are lane 0's, between the warp's barriers and the ticket: it is
+    // lane 0 that publishes the other lanes' partials and sees the other blocks'
     __syncwarp();
     int last = 0;
-    if (l == 0) last = atomicAdd(counter, 1u) == (unsigned)(bpi - 1);
+    if (l == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == (unsigned)(bpi - 1);
+        __threadfence();
+    }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
-    __threadfence();
+    __syncwarp();
     // lane l adds the rows l, l + 32, ..., four rows' loads in flight; the
     // maximum as an integer (the bits of non-negative numbers are in their order,
     // NaN above all), which the FP64 pipe has no part in: an image of a million
