@@ -464,10 +464,12 @@ __device__ __forceinline__ v3<float> local_field_comp(const Stencil<float> &S, c
 // the launch attribute both are no-ops.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisite() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-// The same, and the compiler takes the pointers for new ones after it: loads
+// The same, and the compiler takes the pointers for new ones after it.  Loads
 // through the read-only path (__ldg, const __restrict__) are loads of constant
-// memory to it, which a memory clobber does not hold back, and 20 steps of a film
-// with dipoles came out differently from run to run.
+// memory to it, which a memory clobber does not hold back (20 steps of a film with
+// dipoles came out differently from run to run), and it may take a __restrict__
+// pointer it has not seen handed out for one that no asm statement can write
+// through.
 template <typename P> __device__ __forceinline__ void renew(P &p) { asm volatile("" : "+l"(p)); }
 template <typename... P> __device__ __forceinline__ void wait_prerequisite(P &...p)
 {

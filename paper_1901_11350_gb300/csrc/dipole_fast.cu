@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
     stage_twiddles(tw);
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    wait_prerequisite();  // the spins may come from the pass just before
+    wait_prerequisite(n);  // the spins may come from the pass just before
     float2 a[32];
 #pragma unroll
     for (int n2 = 0; n2 < 16; ++n2) {  // x < 512: the upper half is padding
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(96) k_cols(int n1, float2 *__restrict__ ST, co
         asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         __syncthreads();
     }
-    wait_prerequisite();  // the row spectra
+    wait_prerequisite(ST);  // the row spectra, read through a __restrict__ pointer (see renew)
     float2 *col = ST + ((long)c * 513 + kx) * n1;
     float2 a[32];
 #pragma unroll
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(64 * kRows) k_irows(int n0, int n1, const floa
     float2 *tw = reinterpret_cast<float2 *>(zs + kRows * 512);
     allow_dependents();
     stage_twiddles(tw);
-    wait_prerequisite();  // the column pass's spectra
+    wait_prerequisite(ST);  // the column pass's spectra
     for (int t = threadIdx.x; t < 3 * 513 * kRows; t += blockDim.x) {
         int r = t % kRows, ck = t / kRows;
         if (y0 + r < n1)
