@@ -7,6 +7,7 @@
 #include <cstddef>
 #include <stdint.h>
 
+#include "once_per_device.h"
 #include "spirit_gb.h"
 
 namespace spgb {

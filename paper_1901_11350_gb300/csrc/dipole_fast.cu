@@ -364,19 +364,18 @@ static_assert(3 * kTr >= 3 * 1024, "the transpose tiles must cover the spectra t
 
 cudaError_t dipole_fast_setup()
 {
-    static bool table = false;  // per process
-    if (!table) {
+    static std::atomic<unsigned long long> table{0};
+    cudaError_t e = once_per_device(table, [] {
         float2 tw[32 * 32];
         for (int k2 = 0; k2 < 32; ++k2)
             for (int l = 0; l < 32; ++l) {
                 const double ph = -2.0 * M_PI * (double)(k2 * l) / 1024.0;
                 tw[k2 * 32 + l] = make_float2((float)std::cos(ph), (float)std::sin(ph));
             }
-        cudaError_t e = cudaMemcpyToSymbol(g_tw1024, tw, sizeof tw);
-        if (e != cudaSuccess) return e;
-        table = true;
-    }
-    cudaError_t e = cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem);
+        return cudaMemcpyToSymbol(g_tw1024, tw, sizeof tw);
+    });
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_irows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIrowSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColSmem);

@@ -267,17 +267,12 @@ cudaError_t launch_llg_small(int solver, const Stencil<float> &S, float4 *n, con
     typedef float T;
     if (S.N == 0 || n_steps == 0) return cudaSuccess;
     size_t sm = 3 * sizeof(typename ShRec<T>::type) * (size_t)S.N;
-    static bool attr[3] = {false, false, false};
-    int slot = solver == SP_HEUN ? 0 : (solver == SP_SIB ? 1 : 2);
+    static std::atomic<unsigned long long> done[3];
+    const int slot = solver == SP_HEUN ? 0 : (solver == SP_SIB ? 1 : 2);
     const void *fn = solver == SP_HEUN ? (const void *)k_llg_small<T, SP_HEUN>
                                        : (solver == SP_SIB ? (const void *)k_llg_small<T, SP_SIB>
                                                            : (const void *)k_llg_small<T, SP_DEPONDT>);
-    if (!attr[slot]) {
-        int max_sm = (int)(3 * sizeof(typename ShRec<T>::type) * kSmallMax);
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_sm);
-        if (e != cudaSuccess) return e;
-        attr[slot] = true;
-    }
+    if (cudaError_t e = opt_in_smem(fn, 3 * sizeof(typename ShRec<T>::type) * kSmallMax, done[slot])) return e;
     if (solver == SP_HEUN)
         k_llg_small<T, SP_HEUN><<<1, kSmallThreads, sm, st>>>(S, n, c, n_steps);
     else if (solver == SP_SIB)

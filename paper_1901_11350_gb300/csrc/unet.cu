@@ -21,6 +21,7 @@
 #include <string>
 #include <vector>
 
+#include "once_per_device.h"
 #include "spirit_gb.h"
 #include "spirit_gb_unet.h"
 
@@ -1681,13 +1682,9 @@ template <int BN>
 cudaError_t conv_tc_launch(dim3 grid, const ConvSrc &S, const bf16 *W, const float *bias, int relu, const bf16 *mask,
                            int H, int Wd, int Cout, bf16 *out, cudaStream_t st)
 {
-    static bool attr = false;  // per process; the attribute is per function
     constexpr size_t sm = conv_tc_smem<BN>();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    if (cudaError_t e = spgb::opt_in_smem((const void *)k_conv_tc<BN>, sm, done)) return e;
     k_conv_tc<BN><<<grid, kThreads, sm, st>>>(S, W, bias, relu, mask, H, Wd, Cout, out);
     return cudaGetLastError();
 }
@@ -1696,13 +1693,9 @@ template <int BN>
 cudaError_t conv_ws_launch(dim3 grid, const ConvSrc &S, const bf16 *W, const float *bias, int relu, const bf16 *mask,
                            int H, int Wd, int Cout, bf16 *out, cudaStream_t st)
 {
-    static bool attr = false;
     constexpr size_t sm = conv_ws_smem<BN>();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_ws<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    if (cudaError_t e = spgb::opt_in_smem((const void *)k_conv_ws<BN>, sm, done)) return e;
     k_conv_ws<BN><<<grid, kThreads, sm, st>>>(S, W, bias, relu, mask, H, Wd, Cout, out);
     return cudaGetLastError();
 }
@@ -1732,13 +1725,8 @@ template <int BN>
 cudaError_t conv_halo_launch(int R, const ConvSrc &S, const bf16 *W, const float *bias, int relu, const bf16 *mask,
                              int B, int H, int Wd, int Cout, bf16 *out, cudaStream_t st)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_conv_halo<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHaloSmemMax);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    if (cudaError_t e = spgb::opt_in_smem((const void *)k_conv_halo<BN>, kHaloSmemMax, done)) return e;
     const HaloGeom g = halo_geom(R, Wd, BN);
     dim3 grid((unsigned)(B * (H / R)), (unsigned)(Cout / BN));
     k_conv_halo<BN><<<grid, kThreads, g.smem, st>>>(S, W, bias, relu, mask, H, Wd, Cout, R, out);
@@ -1918,13 +1906,9 @@ template <int BN>
 cudaError_t wgrad_tc_launch(dim3 grid, const ConvSrc &S, const bf16 *dz, int H, int Wd, int Cout, int P, int pps,
                             float *part, float *bias_part, cudaStream_t st)
 {
-    static bool attr = false;  // per process; the attribute is per function
     constexpr size_t sm = wgrad_tc_smem<BN>();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    if (cudaError_t e = spgb::opt_in_smem((const void *)k_wgrad_tc<BN>, sm, done)) return e;
     k_wgrad_tc<BN><<<grid, kThreads, sm, st>>>(S, dz, H, Wd, Cout, P, pps, part, bias_part);
     return cudaGetLastError();
 }
@@ -1933,13 +1917,8 @@ template <int BN>
 cudaError_t wgrad_halo_launch(const WgradHalo &g, const ConvSrc &S, const bf16 *dz, int H, int Wd, int Cout, float *part,
                               float *bias_part, cudaStream_t st)
 {
-    static bool attr = false;  // per process; the attribute is per function
-    if (!attr) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_wgrad_halo<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHaloSmemMax);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    if (cudaError_t e = spgb::opt_in_smem((const void *)k_wgrad_halo<BN>, kHaloSmemMax, done)) return e;
     const dim3 grid((unsigned)((S.C0 + S.C1) / 32), (unsigned)(Cout / BN), (unsigned)g.splits);
     k_wgrad_halo<BN><<<grid, kThreads, wgrad_halo_smem(g.R, Wd, BN), st>>>(S, dz, H, Wd, Cout, g.R, g.bands, g.per, part,
                                                                          bias_part);
