@@ -177,7 +177,6 @@ __device__ __forceinline__ f2sum operator+(f2sum a, f2sum b)
 }
 __device__ __forceinline__ bool operator>(f2sum a, f2sum b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }
 __device__ __forceinline__ f2sum nan_max(f2sum a, f2sum b) { return (a > b || a.hi != a.hi) ? a : b; }
-__device__ __forceinline__ f2sum exact_square(float a) { return {a * a, fmaf(a, a, -(a * a))}; }
 __device__ __forceinline__ f2sum exact_dot(v3<float> a, v3<float> b)
 {
     float p0 = a.x * b.x, p1 = a.y * b.y, p2 = a.z * b.z;

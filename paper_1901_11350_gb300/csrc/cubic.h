@@ -42,6 +42,8 @@ cudaError_t launch_cubic(int pass, int solver, const CubicParams<T> &P, const re
 bool cubic_lean_fits(int nx, int ny, int rows);
 cudaError_t launch_cubic_lean(int pass, const CubicParams<float> &P, const float4 *src, float4 *np, float4 *q,
                               float4 *nout, const LlgConst<float> &c, int per, cudaStream_t st, int rows);
+// CTAs of a lean pass an SM keeps resident (replicas: of the batch's predictor, whose
+// split both passes take)
 int cubic_lean_resident_ctas(int pass, int rows, bool rag, bool replicas);
 // The split of a lean pass without a user's choice: minus the number of runs of
 // planes every column tile is cut into (launch_cubic_lean takes it as `per`).

@@ -611,7 +611,8 @@ cudaError_t lean_launch(int grid, const CubicParams<float> &P, const float4 *src
     auto go = [&](auto kern) {
         return launch_pdl(kern, dim3(grid), dim3(LT), 0, st, P, src, np, q, nout, c, L, G, per);
     };
-    if (llg_reps(c) > 1) return th ? go(k_lean<PASS, DM, TH, R, true, true>) : go(k_lean<PASS, DM, false, R, true, true>);
+    if constexpr (R == 1)  // batches take one column per thread
+        if (llg_reps(c) > 1) return th ? go(k_lean<PASS, DM, TH, 1, true, true>) : go(k_lean<PASS, DM, false, 1, true, true>);
     if (rag) return th ? go(k_lean<PASS, DM, TH, R, true, false>) : go(k_lean<PASS, DM, false, R, true, false>);
     return th ? go(k_lean<PASS, DM, TH, R, false, false>) : go(k_lean<PASS, DM, false, R, false, false>);
 }
@@ -625,12 +626,10 @@ cudaError_t lean_dm(int grid, const CubicParams<float> &P, const float4 *src, fl
     return lean_launch<PASS, 2, R>(grid, P, src, np, q, nout, c, per, st);
 }
 
-template <int PASS, int R> const void *lean_kernel(bool rag, bool repl)
+template <int PASS, int R> const void *lean_kernel(bool rag)
 {
     constexpr bool TH = PASS == 0;
-    return repl ? (const void *)k_lean<PASS, 1, TH, R, true, true>
-                : (rag ? (const void *)k_lean<PASS, 1, TH, R, true, false>
-                       : (const void *)k_lean<PASS, 1, TH, R, false, false>);
+    return rag ? (const void *)k_lean<PASS, 1, TH, R, true, false> : (const void *)k_lean<PASS, 1, TH, R, false, false>;
 }
 
 }  // namespace
@@ -643,7 +642,7 @@ bool cubic_lean_fits(int nx, int ny, int rows)
 cudaError_t launch_cubic_lean(int pass, const CubicParams<float> &P, const float4 *src, float4 *np, float4 *q,
                               float4 *nout, const LlgConst<float> &c, int per, cudaStream_t st, int rows)
 {
-    const int R = rows == 2 ? 2 : 1;
+    const int R = rows == 2 && llg_reps(c) <= 1 ? 2 : 1;
     const long total = cubic_units(P.nx, P.ny, P.nz, R) * llg_reps(c);
     if (total == 0) return cudaSuccess;
     if (per == 0) per = 1;
@@ -699,8 +698,9 @@ int cubic_lean_runs(int nx, int ny, int nz, int rows, int n_rep, int n_sm, int r
 int cubic_lean_resident_ctas(int pass, int rows, bool rag, bool replicas)
 {
     int n = 0;
-    const void *k = rows == 2 ? (pass == 0 ? lean_kernel<0, 2>(rag, replicas) : lean_kernel<1, 2>(rag, replicas))
-                              : (pass == 0 ? lean_kernel<0, 1>(rag, replicas) : lean_kernel<1, 1>(rag, replicas));
+    const void *k = replicas ? (const void *)k_lean<0, 1, true, 1, true, true>
+                    : rows == 2 ? (pass == 0 ? lean_kernel<0, 2>(rag) : lean_kernel<1, 2>(rag))
+                                : (pass == 0 ? lean_kernel<0, 1>(rag) : lean_kernel<1, 1>(rag));
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, LT, 0);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }

@@ -142,7 +142,7 @@ template <typename T> struct Acc {
 template <> struct Acc<float> {
     using type = f2sum;
 };
-// exact_dot and exact_square with products that no addition is fused with
+// exact_dot with products that no addition is fused with
 __device__ __forceinline__ f2sum acc_prod(float a, float b)
 {
     const float p = __fmul_rn(a, b);
@@ -350,10 +350,9 @@ __device__ __forceinline__ void vp_move(rec_t<T> *x, rec_t<T> *v, const rec_t<T>
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_vp_force(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ x,
-                                                     const rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
-                                                     int mode, double *part, unsigned *cnt, double *scal,
-                                                     const int *state)
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1)
+    k_vp_force(const __grid_constant__ Stencil<T> S, const rec_t<T> *__restrict__ x, const rec_t<T> *__restrict__ v,
+               rec_t<T> *__restrict__ F, T dth_m, int mode, double *part, unsigned *cnt, double *scal, const int *state)
 {
     allow_dependents();
     wait_prerequisite(x, v, F, scal, state);  // state, scalars and records come from the kernels before
@@ -872,16 +871,16 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
     int *state = (int *)s->state.p;
     double dth_m = a.dt / (2.0 * a.mass), dt2_2m = a.dt * a.dt / (2.0 * a.mass);
     if (cudaMemsetAsync(state, 0, 4 * sizeof(int), st) != cudaSuccess) return SP_ERR_CUDA;
-    launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F, (T)dth_m, 0, part, cnt,
-               scal, (const int *)state);
+    launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F, (T)dth_m, 0,
+               part, cnt, scal, (const int *)state);
     int k = 0;
     while (k < a.max_iter) {
         int chunk = std::min(a.check_every, a.max_iter - k);
         for (int c = 0; c < chunk; ++c, ++k) {
-            launch_pdl(k_vp_move<T>, dim3(nblk), dim3(kBlock), 0, st, N, x, vv, (const rec_t<T> *)F, (T)a.dt, (T)dt2_2m, a.tol, k,
-                       a.max_iter, (const double *)scal, state);
-            launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F, (T)dth_m,
-                       k == 0 ? 1 : 2, part, cnt, scal, (const int *)state);
+            launch_pdl(k_vp_move<T>, dim3(nblk), dim3(kBlock), 0, st, N, x, vv, (const rec_t<T> *)F, (T)a.dt, (T)dt2_2m,
+                       a.tol, k, a.max_iter, (const double *)scal, state);
+            launch_pdl(k_vp_force<T>, dim3(nblk), dim3(kBlock), 0, st, S, (const rec_t<T> *)x, (const rec_t<T> *)vv, F,
+                       (T)dth_m, k == 0 ? 1 : 2, part, cnt, scal, (const int *)state);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
         if (cudaMemcpyAsync(s->host_state, state, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -909,11 +908,10 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
 // block (tables, state, neighbours, block sum, ticket) with 6 blocks per SM
 // in flight (5: 53, 4: 56).
 template <typename T>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1) k_bvp_force(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img,
-                                                      const Stencil<T> *__restrict__ S, const rec_t<T> *__restrict__ x,
-                                                      const rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m,
-                                                      int mode, double *part, unsigned *cnt, double *scal,
-                                                      const int *state, int *proj)
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SPGB_VP_MINB : 1)
+    k_bvp_force(const BlkInfo *__restrict__ blk, const ImgInfo *__restrict__ img, const Stencil<T> *__restrict__ S,
+                const rec_t<T> *__restrict__ x, const rec_t<T> *__restrict__ v, rec_t<T> *__restrict__ F, T dth_m, int mode,
+                double *part, unsigned *cnt, double *scal, const int *state, int *proj)
 {
     // the tables and stencils do not change while kernels are in flight
     const BlkInfo bi = blk[blockIdx.x];
