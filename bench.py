@@ -61,12 +61,13 @@ CORRECTOR_LAUNCHES = {"heun": 1, "depondt": 1, "sib": 1, "rk4": 3}
 KERNEL_SOURCES = ["paper_1901_11350_gb300/csrc/field_llg.cu", "paper_1901_11350_gb300/csrc/cubic.cu",
                   "paper_1901_11350_gb300/csrc/cubic_lean.cu",
                   "paper_1901_11350_gb300/csrc/common.cuh"]
-# GNEB: bytes per spin and iteration of the method's three passes with FP32
-# records (read n, write g 32; read the three images and g 64; read n, g, v
-# and write n, v 80, plus the per-image reductions' re-reads, about 190) and
-# of this design's four passes (move 80, field 48, tangent 80, force 96)
-GNEB_METHOD_BYTES = 190
-GNEB_DESIGN_BYTES = 304
+# GNEB: bytes per spin and iteration with FP32 records, as this design's passes
+# move them: move reads F and x and writes x (48), field reads x and writes the
+# projected gradient (32), force reads x, the gradient and F and writes F (64);
+# neighbouring images and neighbours come from cache.  No arrangement of the
+# method's passes is known that moves less, so they are its bytes as well.
+GNEB_METHOD_BYTES = 144
+GNEB_DESIGN_BYTES = 144
 
 
 def rank_info():
@@ -466,9 +467,7 @@ def gneb_result(args, compact=False):
                                                  "median": float(np.median(np.abs(bar32 - bar64) / np.abs(bar64)))},
            "setup_s": prep_s}
     # per-iteration roofline over the full batch (GNEB_METHOD_BYTES; the
-    # design's passes move GNEB_DESIGN_BYTES: move 80 (read F, v, x; write v,
-    # x), field 48 (x, next image; write Pg), tangent 80 (three images, Pg;
-    # write tau), force 96 (tau, Pg, F, v; write v, F))
+    # design's passes move GNEB_DESIGN_BYTES)
     import torch
     offs, Ms, ctxs, off = [], [], [], 0
     for ch in chains:
@@ -489,7 +488,7 @@ def gneb_result(args, compact=False):
     it_s = e0.elapsed_time(e1) / 64 / 1e3
     peaks, pk = measured_peaks()
     gbs = GNEB_METHOD_BYTES * off / it_s / 1e9
-    out["roofline"] = {"bound": "hbm", "kernel": "one GNEB iteration of all chains (move, field, tangent, force)",
+    out["roofline"] = {"bound": "hbm", "kernel": "one GNEB iteration of all chains (move, field, coefs, force)",
                        "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
                        "traffic": None, "peak_source": pk, "algorithmic_bytes_per_spin_iteration": GNEB_METHOD_BYTES,
                        "design_bytes_per_spin_iteration": GNEB_DESIGN_BYTES,

@@ -633,7 +633,8 @@ enum {
      * (the batch reads the option of its first chain's context) run in one
      * persistent cooperative launch -- every image of every chain, the
      * passes separated by grid-wide barriers, tangent weights and force
-     * coefficients computed per work block -- instead of one launch per pass
+     * coefficients by a warp per chain in a pass of their own -- instead of one
+     * launch per pass
      * replayed from a CUDA graph; the iterates are bit-identical.  A barrier
      * wait that exceeds SP_OPT_WAIT_LIMIT polls gives up: every block then
      * leaves the kernel, the chain is left part-way through an iteration, and

@@ -17,9 +17,10 @@
 // What bounds the passes is the latency of one wave of few warps (two row
 // blocks per SM, 3.4 columns per SM), so whatever does not depend on the pass
 // before -- the column's Khat and the table of the four-step twiddles, 8 KB in
-// shared memory -- is fetched before the wait for it.  (512 x 512, 40
-// evaluations and steps: 1287 -> 1271 us; and the first call transforms four
-// components on the host instead of six.)
+// shared memory -- is fetched before the wait for it.  (512 x 512, 20 steps with
+// two evaluations each: 1409 us with six components, twiddles from L1 and loads that
+// the compiler could move above the wait; 1355 with four, in turn on one device; and
+// the first call transforms four components on the host instead of six.)
 #include <cmath>
 
 #include "dipole.h"
@@ -203,7 +204,8 @@ __global__ void __launch_bounds__(64 * kRows) k_rows(int n0, int n1, const float
 
 // ------------------------------------------------------------ column pass
 // Block: one column kx, warp c = component.  Khat of the column (6 x 1024
-// reals, structure of arrays) is copied to shared memory with cp.async while
+// reals, 4 x 1024 for a film in the plane, structure of arrays) is copied to
+// shared memory with cp.async while
 // the forward transform over y runs (zero rows y >= n1); product with Khat
 // in the strided layout of the inverse transform's input; rows y < n1
 // written back in place.

@@ -25,10 +25,11 @@
 #endif
 
 // blocks of 256 per SM the FP32 passes' register allocation is held to: with all
-// neighbour loops (512 x 512 hexagonal plane with the dipole field, 20 steps: 6:
-// 1290 us, 5: 1322, 4: 1340; 1024 x 1024 without: 589, 588, 621), and with the loop
-// over the entries alone (512 x 512, 12 bonds, 20 Depondt steps: 8: 447 us, 6: 449;
-// RK4 897 and 911)
+// neighbour loops (512 x 512 hexagonal plane with the dipole field, 20 Depondt
+// steps: 6: 1289 us, 5: 1335, 4: 1344; 1024 x 1024 without: 589, 596, 621; 512 x 512
+// without: 247, 237, 241, SIB 246, 238, 239; two atoms with nine bonds, SIB: 424,
+// 423, 425), and with the loop over the entries alone (512 x 512, 12 bonds, 20
+// Depondt steps: 8: 447 us, 6: 449; RK4 897 and 911)
 #ifndef SPGB_LLG_MINB
 #define SPGB_LLG_MINB 6
 #endif

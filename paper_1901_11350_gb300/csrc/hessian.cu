@@ -137,7 +137,7 @@ __global__ void k_dot_final(const double *__restrict__ part, int nblk, double *_
 // SM -- 6 per spin, vector and step here, 0.7 ms at 128 x 128 spins and 64
 // vectors -- and the chain of three launches a step, each of them four to
 // five dependent accesses to L2 and two FP64 reductions long (9 to 11 us even
-// for one vector).  That run takes 3.1 ms; with a host round trip per
+// for one vector).  That run takes 2.9 ms; with a host round trip per
 // reduction, two passes and a Jacobi diagonalisation on the host it took 16.1.
 constexpr int kLzB = 128;            // spins per tile; threads per block of the per-spin kernels
 constexpr int kLzG = 4;              // groups of kLzB threads in k_lz_dots and k_lz_sub: each takes its share of the

@@ -21,7 +21,7 @@
 // Pg.tau follow from the field pass's products (tau is linear in the weights).
 // 3.6 M spins in 12 chains: 335 -> 240 us an iteration (with tau and v stored,
 // 288 B, and a neighbour loop with indices).  The field pass is 55% of it and
-// bound by the instructions it issues (830 a spin, 61% of the issue slots).
+// bound by the instructions it issues (865 a spin, 65% of the issue slots).
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
@@ -904,7 +904,7 @@ int vp_minimise(MinScratch **sp, const Stencil<T> &S, void *n, void *v, const Mi
 // One image per system.  Per system g: the slots kVF.. from the last force
 // pass, state[2g] iterations moved, state[2g+1] active flag, proj[g] whether
 // the last force pass had a velocity.
-// 1 M spins in 64 systems: 56 -> 52 us an iteration; bound by the chain of a
+// 1 M spins in 64 systems: 56 -> 50 us an iteration; bound by the chain of a
 // block (tables, state, neighbours, block sum, ticket) with 6 blocks per SM
 // in flight (5: 53, 4: 56).
 template <typename T>
