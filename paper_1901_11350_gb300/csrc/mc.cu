@@ -822,8 +822,9 @@ int mc_run(sp_ctx *c, const Stencil<T> &S, void *spins, int n_rep, const double 
             const void *x, *cone, *stats, *temps, *acc, *sw, *part, *cnt, *cosc;
             uint64_t seed;
             double target;
-            int sample, n_rep, prec;
-        } key{x, cone, stats, temps, acc, sw, part, tk, cosc, p->seed, p->target_accept, p->sample, n_rep, (int)sizeof(T)};
+            int sample, n_rep, prec, unused;
+        } key{x, cone, stats, temps, acc, sw, part, tk, cosc, p->seed, p->target_accept, p->sample, n_rep, (int)sizeof(T), 0};
+        static_assert(sizeof(Key) == 9 * sizeof(void *) + 16 + 4 * sizeof(int), "no padding: keys are compared as bytes");
         std::vector<char> gk(sizeof key + sizeof(Stencil<T>));
         memcpy(gk.data(), &key, sizeof key);
         memcpy(gk.data() + sizeof key, &S, sizeof(Stencil<T>));

@@ -39,7 +39,11 @@ struct ImgInfo {
     int N, chain, nu, M, g0, blk0, bpi;
     int kind;  // SP_IMAGE_* or -1: climbing decided by the climbing flag
     int spt;   // spins per thread (GNEB passes; 1 elsewhere)
+    int unused;
 };
+// layouts are compared byte by byte: a padding byte, which holds whatever the stack
+// did, would make an equal one look changed, and its upload cannot be captured
+static_assert(sizeof(ImgInfo) == sizeof(long long) + 10 * sizeof(int), "no padding");
 struct alignas(16) BlkInfo {
     int g, t, chain, ne;  // image, block of the image, the image's chain, its stencil's entries
 };
@@ -969,7 +973,7 @@ int vp_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, const
     for (int c = 0; c < C; ++c) {
         int N = stencils[c].N;
         int bpi = blocks_for(N > 0 ? N : 1);
-        ImgInfo im{spin0[c], N, c, 0, 1, c, (int)blk.size(), bpi, -1, 1};
+        ImgInfo im{spin0[c], N, c, 0, 1, c, (int)blk.size(), bpi, -1, 1, 0};
         for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{c, t, c, stencils[c].off[stencils[c].nb]});
         img.push_back(im);
         total = std::max(total, spin0[c] + (long long)N);
@@ -1071,7 +1075,7 @@ int gneb_batch_run(MinScratch **sp, const std::vector<Stencil<T>> &stencils, con
         int g0 = (int)img.size();
         for (int nu = 0; nu < M[c]; ++nu) {
             int kind = a.kinds ? a.kinds[g0 + nu] : -1;
-            ImgInfo im{spin0[c], N, c, nu, M[c], g0, (int)blk.size(), bpi, kind, spt};
+            ImgInfo im{spin0[c], N, c, nu, M[c], g0, (int)blk.size(), bpi, kind, spt, 0};
             for (int t = 0; t < bpi; ++t) blk.push_back(BlkInfo{(int)img.size(), t, c, stencils[c].off[stencils[c].nb]});
             img.push_back(im);
         }
