@@ -67,15 +67,17 @@ cudaError_t launch_field(const Stencil<T> &S, const rec_t<T> *n, const rec_t<T> 
 template <typename T, Nbr LOOPS, int all> struct LlgMinB {
     static constexpr int value = sizeof(T) == 8 ? 1 : (LOOPS == Nbr::ENTRIES ? SPGB_LLG_MINB_ENTRIES : all);
 };
-// The kernel for a stencil, f(LOOPS).  The loop over the entries alone for one atom
-// per cell in FP32; with several atoms, whose entries differ between neighbouring
-// threads, it gains nothing from more warps (two atoms with nine bonds each, 20
-// Depondt steps: 449 us, 427 with all loops), and FP64 is bound by its pipe (12 bonds:
-// 2826 and 2134 us).
+// The kernel for a stencil, f(LOOPS).  The loop over the entries alone for planes of
+// one atom per cell in FP32 (512 x 512, 12 to 36 bonds: 15% to 25% faster; 100 x 100: 2%
+// to 4%).  In three dimensions it wins and loses (18 and 26 bonds, 20 Depondt steps:
+// 64^3 783 and 1045 us, 723 and 949 with all loops; 128 x 128 x 64 1780 and 2375, 1886
+// and 2502); with several atoms, whose entries differ between neighbouring threads,
+// it gains nothing from more warps (two atoms with nine bonds each: 449 us, 427 with
+// all loops), and FP64 is bound by its pipe (12 bonds: 2826 and 2134 us).
 template <typename T, typename F> auto by_loops(const Stencil<T> &S, F &&f)
 {
     if constexpr (sizeof(T) == 4)
-        if (!S.fixed && S.nb == 1) return f(std::integral_constant<Nbr, Nbr::ENTRIES>{});
+        if (!S.fixed && S.nb == 1 && S.n2 == 1) return f(std::integral_constant<Nbr, Nbr::ENTRIES>{});
     return f(std::integral_constant<Nbr, Nbr::ALL>{});
 }
 

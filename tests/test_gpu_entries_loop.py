@@ -1,5 +1,5 @@
-"""The FP32 passes that hold the loop over a stencil's entries alone: one-atom lattices
-with neither four nor six bonds.
+"""The FP32 passes that hold the loop over a stencil's entries alone: planes of one atom
+per cell with neither four nor six bonds (and a crystal, whose passes hold all loops).
 
 One step of every solver against the oracle (the FP32 bound of one step in
 test_gpu_lean.py), at every kind of edge; and the bits of a batch of lattices,
